@@ -198,36 +198,36 @@ __global__ void __launch_bounds__(kAdjThreads, 1)
         __syncwarp();
     } else if (warp == kAdjMmaWarp) {
         // ------------------------------------------------------------ MMA issue
-        if (lane == 0) {
+        {
+            const uint32_t el = elect_one();
             const uint32_t idesc = idesc_f16(128, 256, BF16);
-            const uint64_t ad0 = desc_sw128(smem_u32(a_base)), bd0 = desc_sw128(smem_u32(b_base));
+            const uint32_t ad0 = warp_uniform(desc_lo(smem_u32(a_base)));
+            const uint32_t bd0 = warp_uniform(desc_lo(smem_u32(b_base)));
+            const uint32_t tm0 = warp_uniform(tmem);
             int slot = 0;
             uint32_t ph = 0;
             bool stop = false;
             for (int li = 0; li < my_items && !stop; ++li) {
                 const int b = li & 1;
                 // the epilogue has read this buffer's previous item (li - 2)
-                if (li >= 2 && !wait_bounded(&acc_empty[b], (uint32_t)((li >> 1) - 1) & 1u, s_abort, err)) break;
-                const uint32_t dt = tmem + (uint32_t)b * 256u;
+                if (li >= 2 && !__all_sync(0xffffffffu, wait_bounded(&acc_empty[b], (uint32_t)((li >> 1) - 1) & 1u,
+                                                                     s_abort, err)))
+                    break;
+                const uint32_t dt = tm0 + (uint32_t)b * 256u;
                 for (int s = 0; s < nst; ++s) {
-                    if (!wait_bounded(&full[slot], ph, s_abort, err)) { stop = true; break; }
+                    if (!__all_sync(0xffffffffu, wait_bounded(&full[slot], ph, s_abort, err))) { stop = true; break; }
                     tc_fence_after();
-                    const uint64_t ad = ad0 + (uint64_t)(slot * (kAdjATile >> 4));
-                    const uint64_t bd = bd0 + (uint64_t)(slot * (kAdjBTile >> 4));
-                    if (s == 0) umma_f16(dt, ad, bd, idesc, 0u);
-                    else umma_f16(dt, ad, bd, idesc, 1u);
-                    umma_f16(dt, ad + 2, bd + 2, idesc, 1u);
-                    umma_f16(dt, ad + 4, bd + 4, idesc, 1u);
-                    umma_f16(dt, ad + 6, bd + 6, idesc, 1u);
-                    umma_commit(&empty[slot]);
-                    if (s == nst - 1) umma_commit(&acc_full[b]);
+                    umma_f16_x4(dt, ad0 + (uint32_t)slot * (kAdjATile >> 4), bd0 + (uint32_t)slot * (kAdjBTile >> 4),
+                                idesc, s ? 1u : 0u, el);
+                    umma_commit_elected(&empty[slot], el);
+                    if (s == nst - 1) umma_commit_elected(&acc_full[b], el);
                     if (++slot == kAdjS) {
                         slot = 0;
                         ph ^= 1u;
                     }
                 }
             }
-            umma_commit(done_bar);
+            umma_commit_elected(done_bar, el);
             wait_bounded(done_bar, 0, &no_abort, err);
         }
         __syncwarp();

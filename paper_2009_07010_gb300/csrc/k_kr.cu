@@ -339,36 +339,38 @@ __global__ void __launch_bounds__(kKrThreads, 1)
         __syncwarp();
     } else if (warp == kKrMmaWarp) {
         // ------------------------------------------------------------ MMA issue
-        if (lane == 0) {
-            // short per-stage issue path (the MMA issue blocks this thread): slot and
-            // phase by increment, descriptors by adding the slot offset to the address
-            // field, constant accumulate flags
-            const uint64_t ad0 = desc_sw128(smem_u32(a_base)), bd0 = desc_sw128(smem_u32(b_base));
+        {
+            // warp-uniform issue path (umma_f16_x4): slot and phase by increment, descriptors
+            // by adding the slot offset to the address field
+            const uint32_t el = elect_one();
+            const uint32_t ad0 = warp_uniform(desc_lo(smem_u32(a_base)));
+            const uint32_t bd0 = warp_uniform(desc_lo(smem_u32(b_base)));
+            const uint32_t tm0 = warp_uniform(tmem);
             int slot = 0, folds = 0;
             uint32_t ph = 0;
             bool stop = false;
             for (int li = 0; !stop; ++li) {
-                const int item = next_item(li, true);
+                int item = next_item(li, lane == 0);
+                __syncwarp();
+                item = __shfl_sync(0xffffffffu, item, 0);
                 if (item < 0) break;
                 const KrItem it = items[item];
-                const int nst = item_stages(it);
-                const uint32_t idesc = idesc_f16(128, it.npx, BF16);
+                const int nst = (int)warp_uniform((uint32_t)item_stages(it));
+                const uint32_t idesc = warp_uniform(idesc_f16(128, it.npx, BF16));
                 int in_acc = 0;
                 for (int s = 0; s < nst; ++s) {
-                    if (!wait_bounded(&full[slot], ph, s_abort, err)) { stop = true; break; }
+                    if (!__all_sync(0xffffffffu, wait_bounded(&full[slot], ph, s_abort, err))) { stop = true; break; }
                     if (in_acc == 0 && folds > 0 &&
-                        !wait_bounded(acc_empty, (uint32_t)(folds - 1) & 1u, s_abort, err)) { stop = true; break; }
+                        !__all_sync(0xffffffffu, wait_bounded(acc_empty, (uint32_t)(folds - 1) & 1u, s_abort, err))) {
+                        stop = true;
+                        break;
+                    }
                     tc_fence_after();
-                    const uint64_t ad = ad0 + (uint64_t)(slot * (kKrATile >> 4));
-                    const uint64_t bd = bd0 + (uint64_t)(slot * (kKrBTile >> 4));
-                    if (in_acc == 0) umma_f16(tmem, ad, bd, idesc, 0u);
-                    else umma_f16(tmem, ad, bd, idesc, 1u);
-                    umma_f16(tmem, ad + 2, bd + 2, idesc, 1u);
-                    umma_f16(tmem, ad + 4, bd + 4, idesc, 1u);
-                    umma_f16(tmem, ad + 6, bd + 6, idesc, 1u);
-                    umma_commit(&empty[slot]);
+                    umma_f16_x4(tm0, ad0 + (uint32_t)slot * (kKrATile >> 4), bd0 + (uint32_t)slot * (kKrBTile >> 4),
+                                idesc, in_acc ? 1u : 0u, el);
+                    umma_commit_elected(&empty[slot], el);
                     if (++in_acc == kKrFoldStages || s == nst - 1) {
-                        umma_commit(acc_full);
+                        umma_commit_elected(acc_full, el);
                         ++folds;
                         in_acc = 0;
                     }
@@ -378,7 +380,7 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                     }
                 }
             }
-            umma_commit(done_bar);
+            umma_commit_elected(done_bar, el);
             wait_bounded(done_bar, 0, &no_abort, err);   // even after an abort (time-limited)
         }
         __syncwarp();

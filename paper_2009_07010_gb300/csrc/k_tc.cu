@@ -518,45 +518,39 @@ __global__ void __launch_bounds__(kThreads, 1)
         // Issuer q takes the stages s = q (mod NISS); with an even ring depth every
         // slot belongs to one issuer.  Accumulation range d covers stages
         // [d kRange, (d + 1) kRange) and uses buffer b = d mod 2.
-        if (lane == 0) {
+        {
             const int q = (warp == kMmaWarp) ? 0 : 1;
-            // The MMA issue blocks this thread until the tensor core takes the
-            // instruction, so the per-stage path is kept short: slot, phase and range
-            // by increment, descriptors by adding the slot offset to the 14-bit address
-            // field (shared addresses < 256 KB cannot carry out of it).
-            const uint32_t idesc = idesc_f16(128, kBMul * ncols, BF16);
-            const uint64_t ad0 = desc_sw128(smem_u32(smem + L.a_off));
-            const uint64_t bd0 = desc_sw128(smem_u32(smem + L.b_off));
+            // The issue path is short and warp-uniform (umma_f16_x4): slot, phase and range
+            // by increment, descriptors by adding the slot offset to the address field.
+            const uint32_t el = elect_one();
+            const uint32_t idesc = warp_uniform(idesc_f16(128, kBMul * ncols, BF16));
+            const uint32_t ad0 = warp_uniform(desc_lo(smem_u32(smem + L.a_off)));
+            const uint32_t bd0 = warp_uniform(desc_lo(smem_u32(smem + L.b_off)));
+            const uint32_t b_units = warp_uniform(b_stage >> 4), tm0 = warp_uniform(tmem);
+            const uint32_t cols = warp_uniform(acc_cols);
             int slot = q, r = q, d = 0;
             uint32_t ph = 0;
             for (int s_i = q; s_i < nst; s_i += NISS) {
-                if (!wait_bounded(&full[slot], ph, s_abort, err)) break;
+                if (!__all_sync(0xffffffffu, wait_bounded(&full[slot], ph, s_abort, err))) break;
                 const int b = d & 1;
                 if (r == q && d >= 2 &&   // first own stage of a range: the buffer's last drain is done
-                    !wait_bounded(&acc_empty[b], (uint32_t)((d >> 1) - 1) & 1u, s_abort, err))
+                    !__all_sync(0xffffffffu,
+                                wait_bounded(&acc_empty[b], (uint32_t)((d >> 1) - 1) & 1u, s_abort, err)))
                     break;
                 tc_fence_after();
-                const uint64_t ad = ad0 + (uint64_t)(slot * (kAStage >> 4));
-                const uint64_t bd = bd0 + (uint64_t)(slot * (b_stage >> 4));
-                const uint32_t dt = tmem + (uint32_t)(2 * q + b) * acc_cols;
-                // K' = 16 per MMA = 32 bytes (descriptor units of 16 B: +2) of the 128-byte row
+                const uint32_t ad = ad0 + (uint32_t)slot * (kAStage >> 4);
+                const uint32_t bd = bd0 + (uint32_t)slot * b_units;
+                const uint32_t dt = tm0 + (uint32_t)(2 * q + b) * cols;
                 // a range's first MMA clears the buffer, except issuer 0's from range 2 on:
                 // the drain has left the compensation of the running sum there
-                if (r == q) umma_f16(dt, ad, bd, idesc, (SPLIT && q == 0 && d >= 2) ? 1u : 0u);
-                else umma_f16(dt, ad, bd, idesc, 1u);
-                umma_f16(dt, ad + 2, bd + 2, idesc, 1u);
-                umma_f16(dt, ad + 4, bd + 4, idesc, 1u);
-                umma_f16(dt, ad + 6, bd + 6, idesc, 1u);
+                umma_f16_x4(dt, ad, bd, idesc, (r != q || (SPLIT && q == 0 && d >= 2)) ? 1u : 0u, el);
                 if (SPLIT) {   // A_hi B_lo, then A_lo B_hi
-                    const uint64_t bl = bd + (uint64_t)(bt_stride >> 4), al = ad + (uint64_t)(kATileBytes >> 4);
-#pragma unroll
-                    for (int kk = 0; kk < 8; kk += 2) umma_f16(dt, ad + kk, bl + kk, idesc, 1u);
-#pragma unroll
-                    for (int kk = 0; kk < 8; kk += 2) umma_f16(dt, al + kk, bd + kk, idesc, 1u);
+                    umma_f16_x4(dt, ad, bd + (bt_stride >> 4), idesc, 1u, el);
+                    umma_f16_x4(dt, ad + (kATileBytes >> 4), bd, idesc, 1u, el);
                 }
-                umma_commit(&empty[slot]);
+                umma_commit_elected(&empty[slot], el);
                 r += NISS;
-                if (r >= kRange || s_i + NISS >= nst) umma_commit(&acc_full[2 * q + b]);
+                if (r >= kRange || s_i + NISS >= nst) umma_commit_elected(&acc_full[2 * q + b], el);
                 if (r >= kRange) {
                     r -= kRange;
                     ++d;
@@ -569,7 +563,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             // all issued MMAs complete before TMEM is released (waited for even after
             // an abort; the wait is still time-limited)
-            umma_commit(&done_bar[q]);
+            umma_commit_elected(&done_bar[q], el);
             wait_bounded(&done_bar[q], 0, &no_abort, err);
         }
         __syncwarp();

@@ -120,6 +120,57 @@ static __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc,
         : "memory");
 }
 
+// Issue path of an MMA warp.  The whole warp runs the issuing loop with warp-uniform
+// control flow and one elected lane executes the tcgen05 instructions under a predicate:
+// descriptors, TMEM address and instruction descriptor then stay in uniform registers and
+// the four K steps of a stage leave back to back.  A loop under `if (lane == 0)` moves
+// every operand to the uniform registers per instruction, one dependent move after
+// another, and among busy generator warps that serial path, not the tensor core, set the
+// stage time (GB300, 16 warps of FP32 and store work beside one issuer: 804 clock cycles
+// per 128 x 256 x 64 stage; 604 in this form; the tensor core alone takes 512.  At
+// 128 x 128 x 64 with idle generators 472 and 300).
+static __device__ __forceinline__ uint32_t elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+// A value that is the same in every lane, marked as such for the compiler.
+static __device__ __forceinline__ uint32_t warp_uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// Low and high words of desc_sw128; the address field (16-byte units) is in the low word,
+// and shared addresses below 256 KB cannot carry out of it.
+static __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
+static constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+
+// The four K = 16 steps (32 bytes of the 128-byte rows each) of one 64-deep operand stage:
+// D (+)= A B^T, the first step accumulating if `accumulate`.  Called by the whole warp;
+// the lane with elected != 0 issues.
+static __device__ __forceinline__ void umma_f16_x4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
+                                                   uint32_t accumulate, uint32_t elected) {
+    asm volatile(
+        "{\n\t.reg .pred p, q, t;\n\t.reg .b32 x, y;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 q, %5, 0;\n\tsetp.eq.u32 t, %6, %6;\n\t"
+        "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
+        "@p tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, q;\n\t"
+        "add.u32 x, %1, 2;\n\tadd.u32 y, %2, 2;\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %3};\n\t"
+        "@p tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+        "add.u32 x, %1, 4;\n\tadd.u32 y, %2, 4;\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %3};\n\t"
+        "@p tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+        "add.u32 x, %1, 6;\n\tadd.u32 y, %2, 6;\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %3};\n\t"
+        "@p tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(b_lo), "r"(kDescHi), "r"(idesc), "r"(accumulate), "r"(elected)
+        : "memory");
+}
+
+// umma_commit by the elected lane of a converged warp.
+static __device__ __forceinline__ void umma_commit_elected(uint64_t *bar, uint32_t elected) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+        "@p tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
+        "r"(elected)
+        : "memory");
+}
+
 // Arrive on `bar` once all previously issued tcgen05.mma of this thread complete.
 static __device__ __forceinline__ void umma_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
