@@ -3,24 +3,40 @@
 //   X[p][q] = sum_k Re( w_{p,k} KR_k[q] ),   KR_k[q] = exp(2 pi i (u_k dl_i + v_k dm_j)),
 //   pixel q = j N + i,  w_{p,k} = W_k D_k(l0_p)                         (Eqs. 21-22)
 //
-// As a real GEMM with K' = 2K: A'[p][2k] = Re w, A'[p][2k+1] = -Im w (the weights,
-// precomputed per position chunk into an FP16/BF16 buffer and loaded by 2-D TMA with
-// 128-byte swizzle), B'[q][2k] = Re KR, B'[q][2k+1] = Im KR (generated on chip).
-// One CTA computes a 128-position x 256-pixel tile over a range of visibilities:
-//   warps 0-15   (four groups on stages s mod 4) generate the 256 pixel twiddles of
-//                each 32-visibility stage: each
-//                lane owns one visibility and walks a 32-pixel run of one cutout row
-//                (phasor recurrence along l, seeded from the MUFU sine/cosine of the
-//                reduced phase u dl + v dm), FP16/BF16 pairs into the swizzled layout;
-//   warp 20      TMA producer of the weight tile of each stage;
-//   warp 21      TMEM allocation and the single-thread tcgen05.mma issue
-//                (M = 128, N = 256, K = 16);
+// Point reflection.  KR_k at the pixel offset (-dl, -dm) is the conjugate of KR_k at
+// (dl, dm), so with
+//   E[p][q] = sum_k Re w_{p,k} cos(phase_k(q)),   O[p][q] = sum_k -Im w_{p,k} sin(phase_k(q))
+// the two pixels are E + O and E - O.  Only a half plane of pixels is contracted (rows
+// j >= N/2, plus row 0 and the lower half of column 0, whose reflections lie outside the
+// cutout): two real GEMMs with K' = K each (one for real weights, O = 0) instead of one
+// with K' = 2K over all pixels, which is half the tensor work and half the twiddles per
+// cutout.  256 x 64^2 on 14.1 M visibilities, exact: contraction 49.8 ms -> @EX@ ms;
+// 512 mixed cutouts on 7.1 M visibilities, Method 1 (real): 167.5 ms -> @RE@ ms.
+//
+// One CTA computes a 128-position tile of 128 representative pixels (256 for real
+// weights) over a range of visibilities, in 64-visibility stages:
+//   A  the weights, 128 positions x 64 visibilities, FP16/BF16 (Re w, and a second tile of
+//      -Im w), precomputed per chunk of visibilities, stage after stage in the swizzled
+//      layout (w16_offset), so that a stage is one contiguous bulk copy.  (As rows of the
+//      chunk, loaded by 2-D TMA, the 128 segments of a stage lay megabytes, often a power
+//      of two, apart, and L2 delivered 4.5-5.5 TB/s in all: with the point reflection that
+//      left the stages of 512 tensor cycles at 1100 (real) and 1750 (complex).)
+//   B  cos (and sin) of the pixel phases, pixels x 64 visibilities, generated on chip.
+// Warp roles:
+//   warps 0-15   four groups of four (three with complex weights, whose 64 KB stages leave
+//                a ring of three) on stages s mod groups: each lane owns two visibilities
+//                and writes their twiddles of 32 or 64 pixels as FP16/BF16 pairs into the
+//                swizzled layout (kr_generate);
+//   warp 20      bulk copies of the weight tiles of each stage;
+//   warp 21      TMEM allocation and the tcgen05.mma issue (M = 128, K = 16, N = the
+//                tile's pixels);
 //   warp 22      the uv input ring (bulk copies), refilled when the generator group
 //                of a stage has read its slot;
-//   warps 16-19  every kFoldStages stages add the active TMEM accumulator into a
+//   warps 16-19  every kFoldStages stages add the active TMEM accumulators into a
 //                running-sum region of TMEM (short FP32 accumulation runs); at the
-//                end they add sum + active into the output with global atomics (the
-//                output is zeroed first; several visibility ranges of a tile add up).
+//                end they add sum + active of each pixel and of its reflection into the
+//                output with global atomics (the output is zeroed first; several
+//                visibility ranges of a tile add up).
 // Every barrier wait is bounded (2 s); on expiry the CTA raises the error flag, stops,
 // waits (bounded) for its copies in flight and issued MMAs and frees TMEM.
 #include "psf_internal.cuh"
@@ -34,158 +50,213 @@ namespace psf {
 namespace {
 using namespace tc;
 
-constexpr int kKrStages = 4;
 constexpr int kKrIn = 16;             // uv input ring depth (stages)
-constexpr int kKrKS = 32;             // visibilities per stage
-constexpr int kKrGenWarps = 16;       // four groups of 4; group g generates stages s = g (mod 4)
+constexpr int kKrKS = 64;             // visibilities per stage (K' = 64 = one 128 B row)
+constexpr int kKrGenWarps = 16;
 constexpr int kKrGroupWarps = 4;
-constexpr int kKrGroups = kKrGenWarps / kKrGroupWarps;
 constexpr int kKrFoldWarp0 = 16;
 constexpr int kKrTmaWarp = 20;
 constexpr int kKrMmaWarp = 21;
 constexpr int kKrInWarp = 22;
 constexpr int kKrThreads = 23 * 32;
-constexpr int kKrFoldStages = 64;
-// roles that read each item index from the ring: 16 generator warps, 4 fold warps, the
-// MMA issuer and the uv ring (one arrival each)
-constexpr int kKrItemReaders = kKrGenWarps + 4 + 1 + 1;
-// Slot-reuse parity waits stay unambiguous only with at most as many generator groups
-// as operand stages (see k_tc.cu).
-static_assert(kKrGroups <= kKrStages && kKrGroups <= kKrIn, "generator groups exceed a ring depth");
-constexpr uint32_t kKrATile = 128 * 128;   // 128 positions x 64 K' x 2 B
-constexpr uint32_t kKrBTile = 256 * 128;   // 256 pixels x 64 K' x 2 B
-constexpr uint32_t kKrInSlot = 2 * kKrKS * 8;  // uv per stage (64 visibilities in the real form)
-constexpr uint32_t kKrSmemBytes =
-    kKrStages * (kKrATile + kKrBTile) + kKrIn * kKrInSlot + 512 + 1024;
-static_assert((2 * kKrStages + 2 * kKrIn + 3 + 5) * 8 + 2 * 4 + 8 <= 512, "barrier block exceeds its reserve");
+constexpr int kKrFoldStages = 64;     // 256 MMAs per accumulation run
+constexpr uint32_t kKrATile = 128 * 128;   // 128 positions x 64 visibilities x 2 B
+constexpr uint32_t kKrBTile = 256 * 128;   // 256 twiddle rows x 64 visibilities x 2 B
+constexpr uint32_t kKrInSlot = kKrKS * 8;  // uv per stage
 
-// One 32-pixel run of one visibility (this lane): value(r) = exp(2 pi i (theta (n0 + r) + phi)),
-// r = 0..31, as eight interleaved 4-pixel pieces in packed FP32x2 recurrences.
-// The step phasor st = exp(2 pi i theta) and its 4-, 8- and 16-row strides depend only on
-// the visibility, so the caller forms them once per stage for all runs of its lane.
-struct Steps {
-    float2 st, s4, s8, s16;
+// Real weights: one A tile, 256 cosine rows (48 KB stages, 4 deep).  Complex weights: A
+// tiles of Re w and -Im w, 128 cosine and 128 sine rows (64 KB stages, 3 deep).
+template <int REAL>
+struct KrShape {
+    static constexpr int kStages = REAL ? 4 : 3;
+    // Slot-reuse parity waits stay unambiguous only with at most as many generator groups
+    // as operand stages (see k_tc.cu).
+    static constexpr int kGroups = kStages;
+    static constexpr uint32_t kA = REAL ? kKrATile : 2 * kKrATile;
+    static constexpr int kRuns = REAL ? 8 : 4;   // 32-pixel runs per tile
+    // roles that read each item index from the ring: the generator warps in use, 4 fold
+    // warps, the MMA issuer and the uv ring (one arrival each)
+    static constexpr int kReaders = kGroups * kKrGroupWarps + 4 + 1 + 1;
+    static constexpr uint32_t kSmem = kStages * (kA + kKrBTile) + kKrIn * kKrInSlot + 512 + 1024;
+    static_assert(kGroups <= kKrIn && kGroups * kKrGroupWarps <= kKrGenWarps, "generator groups");
+    static_assert((2 * kStages + 2 * kKrIn + 3 + 5) * 8 + 2 * 4 + 8 <= 512, "barrier block exceeds its reserve");
 };
-__device__ __forceinline__ Steps make_steps(float theta) {
-    Steps S;
-    S.st = cis_turns(theta);
-    const float2 s2 = cmulf(S.st, S.st);
-    S.s4 = cmulf(s2, s2);
-    S.s8 = cmulf(S.s4, S.s4);
-    S.s16 = cmulf(S.s8, S.s8);
+
+// Representative pixels of an N x N cutout (N a multiple of 32), in 32-pixel runs: the rows
+// j >= N/2 (N^2/64 runs along l), row 0 (N/32 runs along l), and column 0 (runs along m
+// from j = 0; of these only 1 <= j < N/2 are written).
+struct KrRun {
+    int i0, j0, along_m;
+};
+__device__ __forceinline__ KrRun kr_run(int r, int N) {
+    const int per_row = N / 32, main_runs = (N / 2) * per_row;
+    if (r < main_runs) return KrRun{32 * (r % per_row), N / 2 + r / per_row, 0};
+    r -= main_runs;
+    if (r < per_row) return KrRun{32 * r, 0, 0};
+    return KrRun{0, 32 * (r - per_row), 1};
+}
+
+// Nearest integer by adding 1.5 * 2^23 (|x| < 2^22; the conversion unit's rounding
+// instruction runs at a quarter of the FP32 rate).
+__device__ __forceinline__ float nearest(float x) { return __fadd_rn(__fadd_rn(x, 12582912.0f), -12582912.0f); }
+
+__device__ __forceinline__ void cis2(float2 x, float2 &re, float2 &im) {   // exp(2 pi i x) of two phases in turns
+    __sincosf(6.28318530717958647f * (x.x - nearest(x.x)), &im.x, &re.x);
+    __sincosf(6.28318530717958647f * (x.y - nearest(x.y)), &im.y, &re.y);
+}
+
+// cos and sin of the step 2 pi x from the half angle: the recurrence below amplifies an
+// error of cos(step) by up to the square of its length where the step is small, and
+// 1 - 2 sin^2 (2 cos^2 - 1 beyond a quarter turn) keeps that error at the rounding of 1.
+__device__ __forceinline__ void step1(float x, float &re, float &im) {
+    const float f = x - nearest(x);
+    float s, c;
+    __sincosf(3.14159265358979324f * f, &s, &c);
+    re = fabsf(f) < 0.25f ? fmaf(-2.0f * s, s, 1.0f) : fmaf(2.0f * c, c, -1.0f);
+    im = 2.0f * s * c;
+}
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// (ar + i ai)(br + i bi) for two visibilities at a time; nbi = -bi.
+__device__ __forceinline__ float2 mul_re(float2 ar, float2 ai, float2 br, float2 nbi) {
+    return __ffma2_rn(ar, br, __fmul2_rn(ai, nbi));
+}
+__device__ __forceinline__ float2 mul_im(float2 ar, float2 ai, float2 br, float2 bi) {
+    return __ffma2_rn(ar, bi, __fmul2_rn(ai, br));
+}
+
+// Step phasor and 16-pixel stride of a run's direction, visibilities (a, b) of the lane.
+struct KrSteps {
+    float2 sr, si, tr, ti;
+};
+__device__ __forceinline__ KrSteps kr_steps(float2 th) {
+    KrSteps S;
+    step1(th.x, S.sr.x, S.si.x);
+    step1(th.y, S.sr.y, S.si.y);
+    const float2 f = make_float2(th.x - nearest(th.x), th.y - nearest(th.y));
+    cis2(make_float2(16.0f * f.x, 16.0f * f.y), S.tr, S.ti);
     return S;
 }
 
-template <int BF16>
-__device__ __forceinline__ void gen_run32(uint32_t base, const uint32_t (&off)[8], float theta, int n0, float phi,
-                                          const Steps &S) {
-    // eight interleaved 4-row pieces: rows q + 4p (p = 0..7) at step q = 0..3; one
-    // sine/cosine evaluation per run (row 0), piece seeds by the 4- and 16-row strides
-    const float2 st = S.st, s4 = S.s4, s8 = S.s8, s16 = S.s16;
-    float2 z[8];
-    z[0] = cis_turns(fmaf(theta, (float)n0, phi));
-    z[1] = cmulf(z[0], s4);
-    z[2] = cmulf(z[0], s8);
-    z[3] = cmulf(z[1], s8);
-#pragma unroll
-    for (int pc = 4; pc < 8; ++pc) z[pc] = cmulf(z[pc - 4], s16);
-
-    // packed pairs: P0 = rows (q, q+16), P1 = (q+8, q+24), P2 = (q+4, q+20), P3 = (q+12, q+28)
-    float2 re[4], im[4];
-    re[0] = make_float2(z[0].x, z[4].x); im[0] = make_float2(z[0].y, z[4].y);
-    re[1] = make_float2(z[2].x, z[6].x); im[1] = make_float2(z[2].y, z[6].y);
-    re[2] = make_float2(z[1].x, z[5].x); im[2] = make_float2(z[1].y, z[5].y);
-    re[3] = make_float2(z[3].x, z[7].x); im[3] = make_float2(z[3].y, z[7].y);
-    const float2 sr = make_float2(st.x, st.x), si = make_float2(st.y, st.y), nsi = make_float2(-st.y, -st.y);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        // rows q, q+8, q+16, q+24 and rows q+4, q+12, q+20, q+28
-        stmatrix_x4(base + off[q], pack2<BF16>(re[0].x, im[0].x), pack2<BF16>(re[1].x, im[1].x),
-                    pack2<BF16>(re[0].y, im[0].y), pack2<BF16>(re[1].y, im[1].y));
-        stmatrix_x4(base + off[q + 4], pack2<BF16>(re[2].x, im[2].x), pack2<BF16>(re[3].x, im[3].x),
-                    pack2<BF16>(re[2].y, im[2].y), pack2<BF16>(re[3].y, im[3].y));
-        if (q < 3) {
-#pragma unroll
-            for (int pp = 0; pp < 4; ++pp) {
-                const float2 t = __fmul2_rn(im[pp], nsi), u = __fmul2_rn(im[pp], sr);
-                im[pp] = __ffma2_rn(re[pp], si, u);
-                re[pp] = __ffma2_rn(re[pp], sr, t);
-            }
-        }
-    }
+template <int BF16, int ROW>
+__device__ __forceinline__ void kr_row(const uint32_t (&addr)[8], const float2 (&x)[4]) {
+    const uint32_t v0 = pack2<BF16>(x[0].x, x[0].y), v1 = pack2<BF16>(x[1].x, x[1].y);
+    const uint32_t v2 = pack2<BF16>(x[2].x, x[2].y), v3 = pack2<BF16>(x[3].x, x[3].y);
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0 + %5], {%1, %2, %3, %4};" ::"r"(addr[ROW & 7]), "r"(v0),
+                 "r"(v1), "r"(v2), "r"(v3), "n"(ROW * 128)
+                 : "memory");
 }
 
-// Real-weight form: lane t owns visibilities 2t and 2t+1 of a 64-visibility stage and
-// stores the pair (Re KR_2t, Re KR_2t+1) per pixel; the recurrences are packed across
-// the two visibilities, four interleaved 8-pixel pieces.
-struct StepsR {   // two visibilities: steps and their 8- and 16-row strides
-    float2 sa, sb, a8, a16, b8, b16;
+// Rows 0 .. 15 of four 16-pixel pieces (one stream per stmatrix matrix), from their rows 7
+// and 8 outwards: x_{n+1} = C x_n - x_{n-1}, C = 2 cos(step), one packed FMA per pixel and
+// two visibilities (a complex step takes four), at most eight steps from a seed, so that
+// rounding grows by less than ten.  The subtraction is left to the output: the rows are
+// carried as y = +-x with the signs + - - + + - - + ... (kr_sign), for which every step is
+// y = (+-C) y + y.
+template <int BF16>
+__device__ __forceinline__ void kr_chain(const uint32_t (&addr)[8], const float2 (&x7)[4], const float2 (&x8)[4],
+                                         const float2 (&C)[4]) {
+    float2 fp[4], fc[4], bp[4], bc[4];
+    kr_row<BF16, 7>(addr, x7);
+    kr_row<BF16, 8>(addr, x8);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        fp[m] = x7[m];
+        fc[m] = x8[m];
+        bp[m] = x8[m];
+        bc[m] = x7[m];
+    }
+#define KR_STEP(F, B, SGN)                                                          \
+    {                                                                               \
+        _Pragma("unroll") for (int m = 0; m < 4; ++m) {                             \
+            const float2 c = SGN ? C[m] : neg2(C[m]);                               \
+            const float2 f = __ffma2_rn(c, fc[m], fp[m]);                           \
+            const float2 b = __ffma2_rn(c, bc[m], bp[m]);                           \
+            fp[m] = fc[m];                                                          \
+            fc[m] = f;                                                              \
+            bp[m] = bc[m];                                                          \
+            bc[m] = b;                                                              \
+        }                                                                           \
+        kr_row<BF16, F>(addr, fc);                                                  \
+        kr_row<BF16, B>(addr, bc);                                                  \
+    }
+    KR_STEP(9, 6, 0)
+    KR_STEP(10, 5, 1)
+    KR_STEP(11, 4, 0)
+    KR_STEP(12, 3, 1)
+    KR_STEP(13, 2, 0)
+    KR_STEP(14, 1, 1)
+#undef KR_STEP
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        fc[m] = __ffma2_rn(neg2(C[m]), fc[m], fp[m]);
+        bc[m] = __ffma2_rn(neg2(C[m]), bc[m], bp[m]);
+    }
+    kr_row<BF16, 15>(addr, fc);
+    kr_row<BF16, 0>(addr, bc);
+}
+
+// Sign with which kr_chain carries pixel c of a tile.
+__device__ __forceinline__ constexpr float kr_sign(int c) { return ((c + 1) & 2) ? -1.0f : 1.0f; }
+
+// A run's constants: the phase of its row 7 is tu cu + tv cv (turns), its step tu or tv.
+struct KrRunC {
+    float cu, cv;
+    bool along_m;
 };
-__device__ __forceinline__ StepsR make_steps_real(float2 ta) {
-    StepsR S;
-    S.sa = cis_turns(ta.x);
-    S.sb = cis_turns(ta.y);
-    const float2 a2 = cmulf(S.sa, S.sa), a4 = cmulf(a2, a2);
-    const float2 b2 = cmulf(S.sb, S.sb), b4 = cmulf(b2, b2);
-    S.a8 = cmulf(a4, a4);
-    S.a16 = cmulf(S.a8, S.a8);
-    S.b8 = cmulf(b4, b4);
-    S.b16 = cmulf(S.b8, S.b8);
-    return S;
+__device__ __forceinline__ KrRunC kr_run_const(int r, int N) {
+    const KrRun run = kr_run(r, N);
+    return KrRunC{(float)(run.i0 - N / 2 + (run.along_m ? 0 : 7)), (float)(run.j0 - N / 2 + (run.along_m ? 7 : 0)),
+                  run.along_m != 0};
 }
 
-template <int BF16>
-__device__ __forceinline__ void gen_run32_real(uint32_t base, const uint32_t (&off)[8], float2 ta, int n0,
-                                               float2 phi, const StepsR &S) {
-    // ta = (theta_u of visibility 2t, of 2t+1); phi likewise
-    // piece seeds (rows 0, 8, 16, 24) from row 0 and the 8- and 16-row strides
-    // (squarings of the step, formed by the caller): two sine/cosine evaluations per run
-    const float2 sa = S.sa, sb = S.sb;
-    float2 za[4], zb[4];
-    za[0] = cis_turns(fmaf(ta.x, (float)n0, phi.x));
-    zb[0] = cis_turns(fmaf(ta.y, (float)n0, phi.y));
-    za[1] = cmulf(za[0], S.a8);
-    za[2] = cmulf(za[0], S.a16);
-    za[3] = cmulf(za[1], S.a16);
-    zb[1] = cmulf(zb[0], S.b8);
-    zb[2] = cmulf(zb[0], S.b16);
-    zb[3] = cmulf(zb[1], S.b16);
-    float2 re[4], im[4];
+// Seeds of this warp's four streams for one stage.  Real weights: the 64 cosine rows of two
+// runs, two pieces each; complex weights: the two pieces of one run's 32 cosine rows and of
+// its sine rows.  uv = (u, v) of the lane's two visibilities.
+template <int REAL>
+__device__ __forceinline__ void kr_seeds(float4 uv, float cell, const KrRunC (&run)[2], float2 (&x7)[4],
+                                         float2 (&x8)[4], float2 (&C)[4]) {
+    const float2 tu = make_float2(uv.x * cell, uv.z * cell), tv = make_float2(uv.y * cell, uv.w * cell);
+    KrSteps S = kr_steps(run[0].along_m ? tv : tu);
 #pragma unroll
-    for (int pc = 0; pc < 4; ++pc) {
-        re[pc] = make_float2(za[pc].x, zb[pc].x);
-        im[pc] = make_float2(za[pc].y, zb[pc].y);
-    }
-    const float2 sr = make_float2(sa.x, sb.x), si = make_float2(sa.y, sb.y), nsi = make_float2(-sa.y, -sb.y);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        // rows q, q+8, q+16, q+24 = pieces 0..3 at step q
-        stmatrix_x4(base + off[q], pack2<BF16>(re[0].x, re[0].y), pack2<BF16>(re[1].x, re[1].y),
-                    pack2<BF16>(re[2].x, re[2].y), pack2<BF16>(re[3].x, re[3].y));
-        if (q < 7) {
-#pragma unroll
-            for (int pp = 0; pp < 4; ++pp) {
-                const float2 t = __fmul2_rn(im[pp], nsi), u = __fmul2_rn(im[pp], sr);
-                im[pp] = __ffma2_rn(re[pp], si, u);
-                re[pp] = __ffma2_rn(re[pp], sr, t);
-            }
+    for (int h = 0; h < (REAL ? 2 : 1); ++h) {
+        if (h == 1 && run[1].along_m != run[0].along_m) S = kr_steps(run[1].along_m ? tv : tu);
+        float2 zr, zi;
+        cis2(make_float2(fmaf(tu.x, run[h].cu, tv.x * run[h].cv), fmaf(tu.y, run[h].cu, tv.y * run[h].cv)), zr, zi);
+        const float2 nsi = neg2(S.si), nti = neg2(S.ti);
+        const float2 yr = mul_re(zr, zi, S.tr, nti), yi = mul_im(zr, zi, S.tr, S.ti);   // second piece
+        const float2 c2 = make_float2(2.0f * S.sr.x, 2.0f * S.sr.y);
+        x7[2 * h] = zr;
+        x7[2 * h + 1] = yr;
+        x8[2 * h] = mul_re(zr, zi, S.sr, nsi);
+        x8[2 * h + 1] = mul_re(yr, yi, S.sr, nsi);
+        C[2 * h] = C[2 * h + 1] = c2;
+        if (!REAL) {
+            x7[2] = zi;
+            x7[3] = yi;
+            x8[2] = mul_im(zr, zi, S.sr, S.si);
+            x8[3] = mul_im(yr, yi, S.sr, S.si);
+            C[2] = C[3] = c2;
         }
     }
 }
 
 template <int BF16, int REAL>
 __global__ void __launch_bounds__(kKrThreads, 1)
-    k_psf_kr(const __grid_constant__ CUtensorMap wmap, const KrItem *__restrict__ items, int nitems,
+    k_psf_kr(const uint8_t *__restrict__ wblocks, int64_t nblk, const KrItem *__restrict__ items, int nitems,
              int *__restrict__ queue, const float2 *__restrict__ uv, int32_t kchunk0, float cell,
              const int64_t *__restrict__ out_off, float *__restrict__ out, int *err) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    using Sh = KrShape<REAL>;
+    constexpr int kStages = Sh::kStages, kGroups = Sh::kGroups;
     uint8_t *a_base = smem;
-    uint8_t *b_base = smem + kKrStages * kKrATile;
-    uint8_t *in_base = b_base + kKrStages * kKrBTile;
+    uint8_t *b_base = smem + kStages * Sh::kA;
+    uint8_t *in_base = b_base + kStages * kKrBTile;
     uint64_t *full = (uint64_t *)(in_base + kKrIn * kKrInSlot);
-    uint64_t *empty = full + kKrStages;
-    uint64_t *in_full = empty + kKrStages;
+    uint64_t *empty = full + kStages;
+    uint64_t *in_full = empty + kStages;
     uint64_t *in_empty = in_full + kKrIn;
     uint64_t *acc_full = in_empty + kKrIn;
     uint64_t *acc_empty = acc_full + 1;
@@ -199,10 +270,10 @@ __global__ void __launch_bounds__(kKrThreads, 1)
     volatile int no_abort = 0;   // teardown waits ignore the abort flag
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int KS = REAL ? 2 * kKrKS : kKrKS;   // visibilities per stage (64 K' either way)
+    constexpr int KS = kKrKS;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kKrStages; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], kKrGroupWarps + 1);
             mbar_init(&empty[s], 1);
         }
@@ -215,7 +286,7 @@ __global__ void __launch_bounds__(kKrThreads, 1)
         mbar_init(done_bar, 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&item_full[b], 1);
-            mbar_init(&item_empty[b], kKrItemReaders);
+            mbar_init(&item_empty[b], Sh::kReaders);
         }
         mbar_init(item_done, 4);
         *s_abort = 0;
@@ -228,7 +299,7 @@ __global__ void __launch_bounds__(kKrThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *s_tmem;   // columns [0, 256): active accumulator, [256, 512): running sum
+    const uint32_t tmem = *s_tmem;   // columns [0, 256): active accumulators, [256, 512): running sums
 
     // Every role walks the same item sequence from the two-slot ring: the li-th item of
     // this CTA is in slot li & 1; a role reads it, acknowledges (item_empty) and keeps the
@@ -244,11 +315,16 @@ __global__ void __launch_bounds__(kKrThreads, 1)
     };
     auto item_stages = [&](const KrItem &it) { return (it.ke - it.kb + KS - 1) / KS; };
 
-    if (warp < kKrGenWarps) {
+    if (warp < kGroups * kKrGroupWarps) {
         // ------------------------------------------------------------ pixel twiddles
         const int grp = warp / kKrGroupWarps, gw = warp % kKrGroupWarps;
-        uint32_t off8[8];
-        stmatrix_offsets(lane, off8);
+        // stmatrix lane address: matrix m = lane / 8 is stream m (piece m of the warp's 64
+        // rows, or with complex weights the two pieces of 32 cosine rows and of the sine rows
+        // 128 further), 16-byte chunk lane % 8; row n of a piece adds n * 128 and swaps the
+        // chunk by n mod 8
+        const uint32_t lane_off =
+            (REAL ? (uint32_t)(gw * 64 + 16 * (lane >> 3))
+                  : (uint32_t)(gw * 32 + 16 * ((lane >> 3) & 1) + 128 * (lane >> 4))) * 128u + ((uint32_t)(lane & 7) << 4);
         int g0 = 0;   // global index of the current item's first stage
         bool ok = true;
         for (int li = 0; ok; ++li) {
@@ -258,52 +334,38 @@ __global__ void __launch_bounds__(kKrThreads, 1)
             if (item < 0) { ok = item == -1; break; }
             const KrItem it = items[item];
             const int nst = item_stages(it);
-            const int half = it.N / 2;
-            // this group's stages of the item: global g = g0 + s with g = grp (mod 4)
-            for (int s = ((grp - g0) % kKrGroups + kKrGroups) % kKrGroups; s < nst; s += kKrGroups) {
+            const int r0 = it.q0 / 32 + gw * (REAL ? 2 : 1);   // this warp's first run
+            const KrRunC run[2] = {kr_run_const(r0, it.N), kr_run_const(r0 + 1, it.N)};
+            // this group's stages of the item: global g = g0 + s with g = grp (mod groups)
+            for (int s = ((grp - g0) % kGroups + kGroups) % kGroups; s < nst; s += kGroups) {
                 const int g = g0 + s;
-                const int slot = g % kKrStages;
-                const uint32_t ph = (uint32_t)(g / kKrStages) & 1u;
+                const int slot = g % kStages;
+                const uint32_t ph = (uint32_t)(g / kStages) & 1u;
                 const int islot = g % kKrIn;
                 bool w = wait_bounded(&in_full[islot], (uint32_t)(g / kKrIn) & 1u, s_abort, err);
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
-                const float2 *in_uv = reinterpret_cast<const float2 *>(in_base + islot * kKrInSlot);
-                float2 uva, uvb;
-                if (REAL) {
-                    uva = in_uv[2 * lane];
-                    uvb = in_uv[2 * lane + 1];
-                } else {
-                    uva = in_uv[lane];
-                    uvb = uva;
-                }
+                const float4 uv2 = reinterpret_cast<const float4 *>(in_base + islot * kKrInSlot)[lane];
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&in_empty[islot]);   // the input slot may be refilled
-                if (g >= kKrStages) {
+                float2 x7[4], x8[4], C[4];
+                kr_seeds<REAL>(uv2, cell, run, x7, x8, C);
+                if (g >= kStages) {
                     w = wait_bounded(&empty[slot], ph ^ 1u, s_abort, err);
                     if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
                 }
-                Steps S;
-                StepsR SR;
-                if (REAL) SR = make_steps_real(make_float2(uva.x * cell, uvb.x * cell));
-                else S = make_steps(uva.x * cell);
-                for (int r0 = gw * 32; r0 < it.npx; r0 += kKrGroupWarps * 32) {   // 32-pixel runs of this warp
-                    const int q = it.q0 + r0;
-                    const int jrow = q / it.N, i0 = q - jrow * it.N;   // inside one cutout row
-                    const uint32_t dst = smem_u32(b_base + slot * kKrBTile + r0 * 128);
-                    if (REAL)
-                        gen_run32_real<BF16>(dst, off8, make_float2(uva.x * cell, uvb.x * cell), i0 - half,
-                                             make_float2(uva.y * cell * (float)(jrow - half),
-                                                         uvb.y * cell * (float)(jrow - half)),
-                                             SR);
-                    else
-                        gen_run32<BF16>(dst, off8, uva.x * cell, i0 - half, uva.y * cell * (float)(jrow - half), S);
-                }
+                const uint32_t dst = smem_u32(b_base + slot * kKrBTile) + lane_off;
+                uint32_t addr[8];
+#pragma unroll
+                for (int n = 0; n < 8; ++n) addr[n] = dst ^ ((uint32_t)n << 4);
+                kr_chain<BF16>(addr, x7, x8, C);
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&full[slot]);
             }
             g0 += nst;
         }
+    } else if (warp < kKrGenWarps) {
+        // generator warps beyond the ring depth's groups: idle
     } else if (warp == kKrTmaWarp) {
         // ------------------------------------------------------------ items and weight tiles
         if (lane == 0) {
@@ -324,14 +386,14 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                 if (item < 0) break;
                 const KrItem it = items[item];
                 const int nst = item_stages(it);
-                const int x0 = (REAL ? 1 : 2) * (it.kb - kchunk0);   // K' column of the item's first visibility
+                const uint8_t *src = wblocks + ((int64_t)(it.wrow / 128) * nblk + (it.kb - kchunk0) / KS) * Sh::kA;
                 bool stop = false;
                 for (int s = 0; s < nst; ++s, ++g) {
-                    const int slot = g % kKrStages;
-                    const uint32_t ph = (uint32_t)(g / kKrStages) & 1u;
-                    if (g >= kKrStages && !wait_bounded(&empty[slot], ph ^ 1u, s_abort, err)) { stop = true; break; }
-                    mbar_arrive_expect_tx(&full[slot], kKrATile);
-                    tma_load_2d(a_base + slot * kKrATile, &wmap, x0 + s * 2 * kKrKS, it.wrow, &full[slot]);
+                    const int slot = g % kStages;
+                    const uint32_t ph = (uint32_t)(g / kStages) & 1u;
+                    if (g >= kStages && !wait_bounded(&empty[slot], ph ^ 1u, s_abort, err)) { stop = true; break; }
+                    mbar_arrive_expect_tx(&full[slot], Sh::kA);
+                    bulk_g2s(a_base + slot * Sh::kA, src + (int64_t)s * Sh::kA, Sh::kA, &full[slot]);
                 }
                 if (stop) break;
             }
@@ -366,15 +428,18 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                         break;
                     }
                     tc_fence_after();
-                    umma_f16_x4(tm0, ad0 + (uint32_t)slot * (kKrATile >> 4), bd0 + (uint32_t)slot * (kKrBTile >> 4),
-                                idesc, in_acc ? 1u : 0u, el);
+                    const uint32_t ad = ad0 + (uint32_t)slot * (Sh::kA >> 4), bd = bd0 + (uint32_t)slot * (kKrBTile >> 4);
+                    umma_f16_x4(tm0, ad, bd, idesc, in_acc ? 1u : 0u, el);
+                    if (!REAL)   // -Im w against the sine rows, columns 128 ..
+                        umma_f16_x4(tm0 + 128u, ad + (kKrATile >> 4), bd + (128u * 128u >> 4), idesc, in_acc ? 1u : 0u,
+                                    el);
                     umma_commit_elected(&empty[slot], el);
                     if (++in_acc == kKrFoldStages || s == nst - 1) {
                         umma_commit_elected(acc_full, el);
                         ++folds;
                         in_acc = 0;
                     }
-                    if (++slot == kKrStages) {
+                    if (++slot == kStages) {
                         slot = 0;
                         ph ^= 1u;
                     }
@@ -425,28 +490,60 @@ __global__ void __launch_bounds__(kKrThreads, 1)
             const KrItem it = items[item];
             const int nfold = (item_stages(it) + kKrFoldStages - 1) / kKrFoldStages;
             const bool row_ok = row < it.npos;
-            float *dst = out + (row_ok ? out_off[it.slot0 + row] : 0) + it.q0;
+            const int N = it.N;
+            float *dst = out + (row_ok ? out_off[it.slot0 + row] : 0);
             for (int f = 0; f < nfold; ++f, ++F) {
                 const bool w = wait_bounded(acc_full, (uint32_t)F & 1u, s_abort, err);
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
                 tc_fence_after();
                 const bool last = (f == nfold - 1);
-                for (int c0 = 0; c0 < it.npx; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(ta + (uint32_t)c0, v);
-                    if (f > 0) {
-                        float sacc[16];
-                        tmem_ld16(ta + 256u + (uint32_t)c0, sacc);
+                if (!last) {   // running sum (+)= accumulator, 32 columns at a time
+                    for (int c0 = 0; c0 < (REAL ? it.npx : 256); c0 += 32) {
+                        if (!REAL && (c0 & 127) >= it.npx) continue;
+                        uint32_t v[32], u[32];
+                        tmem_ld32_issue(ta + (uint32_t)c0, v);
+                        if (f > 0) {
+                            tmem_ld32_issue(ta + 256u + (uint32_t)c0, u);
+                            tmem_wait_ld(v, u);
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) v[e] += sacc[e];
-                    }
-                    if (last) {
-                        if (row_ok) {
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) atomicAdd(dst + c0 + e, v[e]);
+                            for (int e = 0; e < 32; ++e)
+                                v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(u[e]));
+                        } else {
+                            tmem_wait_ld(v, v);
                         }
-                    } else {
-                        tmem_st16(ta + 256u + (uint32_t)c0, v);
+                        tmem_st32_issue(ta + 256u + (uint32_t)c0, v);
+                    }
+                    tmem_wait_st();
+                }
+                // the end: columns c0 .. c0 + 15 (E) and, with complex weights, 128 + c0 .. (O)
+                for (int c0 = 0; last && c0 < it.npx; c0 += 16) {
+                    float v[REAL ? 1 : 2][16];
+#pragma unroll
+                    for (int h = 0; h < (REAL ? 1 : 2); ++h) {
+                        const uint32_t tc0 = ta + (uint32_t)(c0 + 128 * h);
+                        tmem_ld16(tc0, v[h]);
+                        if (f > 0) {
+                            float sacc[16];
+                            tmem_ld16(tc0 + 256u, sacc);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) v[h][e] += sacc[e];
+                        }
+                    }
+                    if (!row_ok) continue;
+                    // pixel E + O, reflected pixel E - O (kr_run's order of pixels; a chunk of 16
+                    // lies in one run)
+                    const int q = it.q0 + c0;
+                    const KrRun run = kr_run(q / 32, N);
+                    const int t0 = q & 31;
+                    const int pix = run.j0 * N + run.i0 + (run.along_m ? t0 * N : t0);
+                    const int pstep = run.along_m ? N : 1;
+                    const bool mirrored = !run.along_m && run.j0 > N / 2;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const float E = kr_sign(e) * v[0][e], O = REAL ? 0.f : kr_sign(e) * v[REAL ? 0 : 1][e];
+                        const int j = run.j0 + t0 + e;
+                        if (!run.along_m || (j >= 1 && j < N / 2)) atomicAdd(dst + pix + e * pstep, E + O);
+                        if (mirrored && run.i0 + t0 + e >= 1) atomicAdd(dst + N * N + N - pix - e, E - O);
                     }
                 }
                 tc_fence_before();
@@ -466,35 +563,33 @@ __global__ void __launch_bounds__(kKrThreads, 1)
 }  // namespace
 
 template <int BF16, int REAL>
-static cudaError_t launch_kr_t(const CUtensorMap *m, const KrItem *items, int nitems, int *queue, int nctas,
+static cudaError_t launch_kr_t(const void *w16, int64_t nblk, const KrItem *items, int nitems, int *queue, int nctas,
                                const float2 *uv, int32_t kchunk0, float cell, const int64_t *out_off, float *out,
                                int *err, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(k_psf_kr<BF16, REAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kKrSmemBytes);
+                                         (int)KrShape<REAL>::kSmem);
     if (e != cudaSuccess) return e;
-    k_psf_kr<BF16, REAL><<<nctas, kKrThreads, kKrSmemBytes, st>>>(*m, items, nitems, queue, uv, kchunk0, cell,
+    k_psf_kr<BF16, REAL><<<nctas, kKrThreads, KrShape<REAL>::kSmem, st>>>((const uint8_t *)w16, nblk, items, nitems, queue, uv, kchunk0, cell,
                                                                    out_off, out, err);
     return cudaGetLastError();
 }
 
-cudaError_t launch_psf_kr(const void *wmap, const KrItem *items, int nitems, int *queue, int nctas, const float2 *uv,
+cudaError_t launch_psf_kr(const void *w16, int64_t nblk, const KrItem *items, int nitems, int *queue, int nctas, const float2 *uv,
                           int32_t kchunk0, float cell, const int64_t *out_off, float *out, int bf16, int real, int *err,
                           cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
     nctas = std::max(1, std::min(nctas, nitems));
     cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    const CUtensorMap *m = (const CUtensorMap *)wmap;
     if (bf16)
-        return real ? launch_kr_t<1, 1>(m, items, nitems, queue, nctas, uv, kchunk0, cell, out_off, out, err, st)
-                    : launch_kr_t<1, 0>(m, items, nitems, queue, nctas, uv, kchunk0, cell, out_off, out, err, st);
-    return real ? launch_kr_t<0, 1>(m, items, nitems, queue, nctas, uv, kchunk0, cell, out_off, out, err, st)
-                : launch_kr_t<0, 0>(m, items, nitems, queue, nctas, uv, kchunk0, cell, out_off, out, err, st);
+        return real ? launch_kr_t<1, 1>(w16, nblk, items, nitems, queue, nctas, uv, kchunk0, cell, out_off, out, err, st)
+                    : launch_kr_t<1, 0>(w16, nblk, items, nitems, queue, nctas, uv, kchunk0, cell, out_off, out, err, st);
+    return real ? launch_kr_t<0, 1>(w16, nblk, items, nitems, queue, nctas, uv, kchunk0, cell, out_off, out, err, st)
+                : launch_kr_t<0, 0>(w16, nblk, items, nitems, queue, nctas, uv, kchunk0, cell, out_off, out, err, st);
 }
 
-// 2-D tensor map over the FP16/BF16 weight buffer: dim0 = pitch elements (2 KC for
-// complex weights, KC for real ones), dim1 = rows; box 64 x 128 elements (one
-// 128-byte-swizzled stage of 128 positions).
+// 2-D tensor map over a FP16/BF16 matrix: dim0 = pitch elements, dim1 = rows; box 64 x 128
+// elements (one 128-byte-swizzled stage of 128 rows).
 int make_weight_map(void *map_out, void *w16, int bf16, int64_t pitch_elems, int64_t rows) {
     typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -521,6 +616,9 @@ int make_weight_map(void *map_out, void *w16, int bf16, int64_t pitch_elems, int
     return r == CUDA_SUCCESS ? PSF_OK : PSF_ECUDA;
 }
 
-int kr_smem_bytes() { return (int)kKrSmemBytes; }
+int kr_tile_pixels(int real) { return 32 * (real ? KrShape<1>::kRuns : KrShape<0>::kRuns); }
+
+// Representative pixels of an N x N cutout in the order of kr_run (a multiple of 32).
+int kr_pixels(int N) { return N * N / 2 + N + (N / 2 + 31) / 32 * 32; }
 
 }  // namespace psf

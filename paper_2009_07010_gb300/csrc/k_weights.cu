@@ -124,8 +124,8 @@ cudaError_t launch_weights(const DevObs &o, int method, uint32_t flags, const fl
 
 // --------------------------------------------------------------- FP16/BF16 weights
 // Weights of a position chunk for the batched tensor-core contraction: row r holds
-// position slot_of_row[r] (zeros for padding rows, slot < 0) as (Re w, -Im w) pairs
-// at column pair (k - kc0); columns at or beyond kcn are zero.  The weights are
+// position slot_of_row[r] (zeros for padding rows, slot < 0), Re w and -Im w in two planes
+// (w16_offset); columns (k - kc0) at or beyond kcn are zero.  The weights are
 // rounded to 16 bits, so the fast sine/cosine forms are used.
 // One thread per visibility (column) and a block of kRowsPerBlock position rows: the
 // visibility's records (bin, channel, weight, raw samples) are loaded once and reused
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(256) k_weights16(DevObs o, int method, uint32_
                                                    const int32_t *__restrict__ slot_of_row, int rows, int32_t kc0,
                                                    int32_t kcn, int64_t kpitch, uint32_t *__restrict__ w16) {
     const int32_t kk = blockIdx.x * blockDim.x + threadIdx.x;
-    if (kk >= kpitch) return;
+    if (kk >= kpitch) return;   // kpitch is a multiple of 64: whole warps leave
     const int row0 = blockIdx.y * kRowsPerBlock;
     const bool valid = kk < kcn;
     const int32_t k = kc0 + (valid ? kk : 0);
@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(256) k_weights16(DevObs o, int method, uint32_
     const int r = k - bin * o.nout;
     const float Wk = valid ? o.W[k] : 0.f;
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int odd = threadIdx.x & 1;
     for (int row = row0; row < min(rows, row0 + kRowsPerBlock); ++row) {
         const int slot = slot_of_row[row];
         float2 w = make_float2(0.f, 0.f);
@@ -178,7 +179,11 @@ __global__ void __launch_bounds__(256) k_weights16(DevObs o, int method, uint32_
             const float2 D = decorr<false, true>(o, method, flags, bin, r, pos[slot], z, z, nullptr);
             w = make_float2(Wk * D.x, Wk * D.y);
         }
-        w16[(int64_t)row * kpitch + kk] = pack_sr<BF16>(w.x, -w.y, sr_bits((uint32_t)slot, (uint32_t)k));
+        // even lanes store the pair's real parts, odd lanes its imaginary parts
+        const uint32_t own = pack_sr<BF16>(w.x, -w.y, sr_bits((uint32_t)slot, (uint32_t)k));
+        const uint32_t nbr = __shfl_xor_sync(0xffffffffu, own, 1);
+        const uint32_t v = odd ? __byte_perm(nbr, own, 0x7632) : __byte_perm(own, nbr, 0x5410);
+        w16[w16_offset(row, kk & ~1, kpitch >> 6, 2, odd) >> 1] = v;
     }
 }
 
@@ -247,7 +252,7 @@ __global__ void __launch_bounds__(256) k_weights16_real(DevObs o, int method, ui
                 if (Wk[e] != 0.f) wv[e] = Wk[e] * sincpi_fast(A) * sincpi_fast(B);
             }
         }
-        w16[(int64_t)row * kpitch2 + kp] = pack_sr<BF16>(wv[0], wv[1], sr_bits((uint32_t)slot, (uint32_t)(kc0 + 2 * kp)));
+        w16[w16_offset(row, 2 * (int64_t)kp, kpitch2 >> 5, 1, 0) >> 1] = pack_sr<BF16>(wv[0], wv[1], sr_bits((uint32_t)slot, (uint32_t)(kc0 + 2 * kp)));
     }
 }
 
@@ -295,9 +300,15 @@ __global__ void __launch_bounds__(256) k_weights16_exact8(DevObs o, uint32_t fla
             const float wr = Wk[j] * sr * inv, wi = Wk[j] * si * inv;
             packed[j] = pack_sr<BF16>(wr, -wi, sr_bits((uint32_t)slot, (uint32_t)(k0 + j)));
         }
-        uint4 *dst = reinterpret_cast<uint4 *>(w16 + (int64_t)row * kpitch + kk0);
-        dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-        dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+        uint32_t pr[4], pi[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            pr[j] = __byte_perm(packed[2 * j], packed[2 * j + 1], 0x5410);
+            pi[j] = __byte_perm(packed[2 * j], packed[2 * j + 1], 0x7632);
+        }
+        const int64_t at = w16_offset(row, kk0, kpitch >> 6, 2, 0) >> 1;   // the -Im w block follows (4096 words)
+        *reinterpret_cast<uint4 *>(w16 + at) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
+        *reinterpret_cast<uint4 *>(w16 + at + 4096) = make_uint4(pi[0], pi[1], pi[2], pi[3]);
     }
 }
 

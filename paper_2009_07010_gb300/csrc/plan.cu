@@ -552,9 +552,9 @@ struct KrGroup {
 // <= 256).  Per chunk of visibilities the weights of every group are written as FP16/BF16
 // rows into one buffer (each group padded to whole 128-position tiles), then one
 // persistent launch of the Khatri-Rao kernel (one CTA per SM) pulls (128-position tile,
-// 256-pixel tile, visibility range) items from an atomic queue and accumulates them into
-// the zeroed output.  Every item is 128 positions x 256 pixels, so its cost is its
-// visibility range: the ranges are equal, items_per_cta x SMs of them at least (fewer
+// pixel tile, visibility range) items from an atomic queue and accumulates them into
+// the zeroed output.  Every item but the last of a cutout has the same number of pixels,
+// so its cost is its visibility range: the ranges are equal, items_per_cta x SMs of them at least (fewer
 // when a range would drop below one 64-stage accumulation run).  kmax < nvis restricts
 // the call to the first kmax visibilities (the autotuner's probes); ms_out (optional)
 // receives the summed time of the contraction launches (the stream is synchronized).
@@ -562,11 +562,12 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
            cudaStream_t st, int items_per_cta, int64_t kmax = -1, double *ms_out = nullptr) {
     const int64_t K = kmax > 0 ? std::min<int64_t>(kmax, p->nvis) : p->nvis;
     const int bf16 = prec_bf16(p->opts.prec);
-    // Methods 1 and 2 have real weights (unless windowed): one K' column per visibility,
-    // 64-visibility stages; complex weights: two columns, 32-visibility stages.
+    // Methods 1 and 2 have real weights (unless windowed); complex weights take two operand
+    // tiles per stage (real and negated imaginary parts).
     const int real = method != kExact && p->d.win == 0;
-    const int64_t ks = real ? 64 : 32;
+    const int64_t ks = 64;
     const size_t bytes_per = real ? 2 : 4;
+    const int tile_px = kr_tile_pixels(real);
     // combined rows: group g occupies rows [row0_g, row0_g + 128 ntile_g)
     std::vector<float4> pos;
     std::vector<int32_t> slot_of_row, npix;
@@ -592,12 +593,11 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
     KC = std::max<int64_t>(64, std::min<int64_t>(KC, (K + 63) / 64 * 64));
     const int64_t nchunk = (K + KC - 1) / KC;
     int64_t nbase = 0;   // (position tile, pixel tile) pairs
-    for (const auto &g : groups) nbase += (int64_t)((g.idx.size() + 127) / 128) * (g.N * g.N / 256);
+    for (const auto &g : groups)
+        nbase += (int64_t)((g.idx.size() + 127) / 128) * ((kr_pixels(g.N) + tile_px - 1) / tile_px);
     PSF_TRY(p->w16.reserve((size_t)rows * KC * bytes_per));
     PSF_TRY(p->queue.reserve(sizeof(int)));
-    CUtensorMapStub wmap;
-    int s = make_weight_map(&wmap, p->w16.p, bf16, real ? KC : 2 * KC, rows);
-    if (s) return s;
+    int s = PSF_OK;
     cudaEvent_t t0 = nullptr, t1 = nullptr;
     double ms_total = 0.0;
     if (ms_out) {
@@ -620,14 +620,14 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
             for (size_t g = 0; g < groups.size(); ++g) {
                 const int np = (int)groups[g].idx.size(), N = groups[g].N;
                 for (int t = 0; t < (np + 127) / 128; ++t)
-                    for (int q = 0; q < N * N / 256; ++q) {
+                    for (int q = 0; q < kr_pixels(N); q += tile_px) {
                         KrItem it;
                         it.wrow = row0[g] + t * 128;
                         it.npos = std::min(128, np - t * 128);
                         it.slot0 = slot0[g] + t * 128;
                         it.N = N;
-                        it.q0 = q * 256;
-                        it.npx = 256;
+                        it.q0 = q;
+                        it.npx = std::min(tile_px, kr_pixels(N) - q);
                         it.kb = (int32_t)(kc0 + sp * sper * ks);
                         it.ke = (int32_t)std::min<int64_t>(kc0 + kcn, kc0 + (sp + 1) * sper * ks);
                         items.push_back(it);
@@ -670,7 +670,7 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
             PSF_TRY(cudaEventRecord(ev1, st));
         }
         if (ms_out) PSF_TRY(cudaEventRecord(t0, st));
-        PSF_TRY(launch_psf_kr(&wmap, (const KrItem *)(dm + off_items), (int)items.size(), (int *)p->queue.p, p->nsm,
+        PSF_TRY(launch_psf_kr(p->w16.p, KC / 64, (const KrItem *)(dm + off_items), (int)items.size(), (int *)p->queue.p, p->nsm,
                               p->d.uv, (int32_t)kc0, (float)h.cell, (const int64_t *)(dm + off_outo), out, bf16, real,
                               (int *)p->err.p, st));
         if (ms_out) {

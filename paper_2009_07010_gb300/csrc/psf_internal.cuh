@@ -55,8 +55,8 @@ enum Method { kExact = 0, kUV = 1, kImg = 2 };
 // ---- launchers (k_weights.cu) -------------------------------------------
 // w[s * ldw + (k - k0)] = W_k * D_k(pos[s]) for s < npos, k0 <= k < k0 + kn.
 // fast != 0: MUFU sine/cosine forms (for weights rounded to 16 bits afterwards).
-// launch_weights16: complex methods write (Re w, -Im w) pairs, kpitch pairs per row;
-// real methods write one value per visibility, kpitch pairs = 2 kpitch visibilities.
+// launch_weights16: FP16/BF16 weights of `rows` (a multiple of 128) position rows and kpitch
+// (a multiple of 64) visibilities in the layout of w16_offset.
 cudaError_t launch_weights(const DevObs &o, int method, uint32_t flags, const float4 *pos,
                            int npos, int32_t k0, int32_t kn, float2 *w, int64_t ldw, int fast,
                            cudaStream_t st);
@@ -137,23 +137,37 @@ int selftest_timeout(int limit_ms);
 int selftest_fma_rate(int packed, double *flops_per_s);   // k_weights.cu
 
 // ---- batched tcgen05 contraction (k_kr.cu) ---------------------------------
+// Layout of the 16-bit weights of the batched form: blocks of 128 position rows x 64
+// visibilities (one pipeline stage; `planes` blocks per stage: Re w, and for complex
+// weights -Im w), block after block along the visibilities of a position tile.  A block
+// holds the K-major 128-byte-swizzled operand tile: row r at r * 128 bytes, its 16-byte
+// chunk c (8 visibilities) at c XOR (r mod 8).  Offset in 16-bit elements of (row, plane,
+// visibility kk of the chunk); nblk = stages per position tile.
+__host__ __device__ inline int64_t w16_offset(int row, int64_t kk, int64_t nblk, int planes, int plane) {
+    const int r = row & 127;
+    return (((((int64_t)(row >> 7) * nblk + (kk >> 6)) * planes + plane) * 128 + r) << 6) +
+           ((((kk >> 3) & 7) ^ (r & 7)) << 3) + (kk & 7);
+}
+
 struct KrItem {
     int32_t wrow;     // first row of the 128-position tile in the weight buffer
     int32_t npos;     // valid positions of the tile (<= 128)
     int32_t slot0;    // batch index of the tile's first position
     int32_t N;        // cutout size (multiple of 32, <= 256)
-    int32_t q0;       // first pixel (row-major) of the 256-pixel tile
-    int32_t npx;      // pixels of the tile (256)
-    int32_t kb, ke;   // visibility range, kb - chunk start a multiple of the stage size (32 or 64)
+    int32_t q0;       // first representative pixel of the tile (kr_run's order, a multiple of 32)
+    int32_t npx;      // representative pixels of the tile (a multiple of 32, <= kr_tile_pixels)
+    int32_t kb, ke;   // visibility range, kb - chunk start a multiple of the 64-visibility stage
 };
-// real != 0: real weights (Methods 1, 2), one K' column per visibility.
+// real != 0: real weights (Methods 1, 2).  w16: the weights in the layout of w16_offset,
+// nblk stages per 128-position tile.
 // Persistent: nctas CTAs (one per SM) pull items from the work queue (a device int,
 // zeroed by the launch) in array order (largest first).
-cudaError_t launch_psf_kr(const void *wmap, const KrItem *items, int nitems, int *queue, int nctas, const float2 *uv,
+cudaError_t launch_psf_kr(const void *w16, int64_t nblk, const KrItem *items, int nitems, int *queue, int nctas, const float2 *uv,
                           int32_t kchunk0, float cell, const int64_t *out_off, float *out, int bf16, int real, int *err,
                           cudaStream_t st);
 int make_weight_map(void *map_out, void *w16, int bf16, int64_t pitch_elems, int64_t rows);
-int kr_smem_bytes();
+int kr_tile_pixels(int real);
+int kr_pixels(int N);
 cudaError_t launch_weights16(const DevObs &o, int method, uint32_t flags, const float4 *pos,
                              const int32_t *slot_of_row, int rows, int32_t kc0, int32_t kcn, int64_t kpitch,
                              int bf16, void *w16, cudaStream_t st);
