@@ -10,8 +10,9 @@
 // j >= N/2, plus row 0 and the lower half of column 0, whose reflections lie outside the
 // cutout): two real GEMMs with K' = K each (one for real weights, O = 0) instead of one
 // with K' = 2K over all pixels, which is half the tensor work and half the twiddles per
-// cutout.  256 x 64^2 on 14.1 M visibilities, exact: contraction 49.8 ms -> @EX@ ms;
-// 512 mixed cutouts on 7.1 M visibilities, Method 1 (real): 167.5 ms -> @RE@ ms.
+// cutout.  256 x 64^2 on 14.1 M visibilities, exact: contraction 49.8 ms -> 22 ms;
+// 512 mixed cutouts on 7.1 M visibilities, Method 1 (real): 167.5 ms -> 58 ms
+// (both with the contiguous weight stages and the unrolled issue loop below).
 //
 // One CTA computes a 128-position tile of 128 representative pixels (256 for real
 // weights) over a range of visibilities, in 64-visibility stages:
@@ -23,20 +24,23 @@
 //      left the stages of 512 tensor cycles at 1100 (real) and 1750 (complex).)
 //   B  cos (and sin) of the pixel phases, pixels x 64 visibilities, generated on chip.
 // Warp roles:
-//   warps 0-15   four groups of four (three with complex weights, whose 64 KB stages leave
-//                a ring of three) on stages s mod groups: each lane owns two visibilities
-//                and writes their twiddles of 32 or 64 pixels as FP16/BF16 pairs into the
-//                swizzled layout (kr_generate);
+//   generators   one group of four warps per operand slot (warps 0-15, or 0-11 with complex
+//                weights, whose 64 KB stages leave a ring of three): each lane owns two
+//                visibilities of a stage and writes their twiddles of 32 or 64 pixels as
+//                FP16/BF16 pairs into the swizzled layout (kr_seeds, kr_chain);
+//   fold warps   (the others up to 19) every fold range add the active TMEM accumulators into
+//                a running-sum region of TMEM (short FP32 accumulation runs); at the end they
+//                add sum + active of each pixel and of its reflection into the output with
+//                global atomics (the output is zeroed first; several visibility ranges of a
+//                tile add up);
 //   warp 20      bulk copies of the weight tiles of each stage;
-//   warp 21      TMEM allocation and the tcgen05.mma issue (M = 128, K = 16, N = the
-//                tile's pixels);
+//   warp 21      TMEM allocation and the tcgen05.mma issue (M = 128, K = 16, N = the tile's
+//                pixels).  Among the generators its instructions, not the tensor core, set
+//                the stage time (without generators a real stage takes 585 cycles, without
+//                MMAs 730, together 812), so its loop is unrolled over the ring slots;
 //   warp 22      the uv input ring (bulk copies), refilled when the generator group
-//                of a stage has read its slot;
-//   warps 16-19  every kFoldStages stages add the active TMEM accumulators into a
-//                running-sum region of TMEM (short FP32 accumulation runs); at the
-//                end they add sum + active of each pixel and of its reflection into the
-//                output with global atomics (the output is zeroed first; several
-//                visibility ranges of a tile add up).
+//                of a stage has read its slot.
+// An item starts in operand slot 0; barrier phases are kept per slot.
 // Every barrier wait is bounded (2 s); on expiry the CTA raises the error flag, stops,
 // waits (bounded) for its copies in flight and issued MMAs and frees TMEM.
 #include "psf_internal.cuh"
@@ -52,14 +56,11 @@ using namespace tc;
 
 constexpr int kKrIn = 16;             // uv input ring depth (stages)
 constexpr int kKrKS = 64;             // visibilities per stage (K' = 64 = one 128 B row)
-constexpr int kKrGenWarps = 16;
 constexpr int kKrGroupWarps = 4;
-constexpr int kKrFoldWarp0 = 16;
 constexpr int kKrTmaWarp = 20;
 constexpr int kKrMmaWarp = 21;
 constexpr int kKrInWarp = 22;
 constexpr int kKrThreads = 23 * 32;
-constexpr int kKrFoldStages = 64;     // 256 MMAs per accumulation run
 constexpr uint32_t kKrATile = 128 * 128;   // 128 positions x 64 visibilities x 2 B
 constexpr uint32_t kKrBTile = 256 * 128;   // 256 twiddle rows x 64 visibilities x 2 B
 constexpr uint32_t kKrInSlot = kKrKS * 8;  // uv per stage
@@ -68,17 +69,21 @@ constexpr uint32_t kKrInSlot = kKrKS * 8;  // uv per stage
 // tiles of Re w and -Im w, 128 cosine and 128 sine rows (64 KB stages, 3 deep).
 template <int REAL>
 struct KrShape {
-    static constexpr int kStages = REAL ? 4 : 3;
-    // Slot-reuse parity waits stay unambiguous only with at most as many generator groups
-    // as operand stages (see k_tc.cu).
-    static constexpr int kGroups = kStages;
+    static constexpr int kStages = REAL ? 4 : 3;    // one generator group per slot
+    static constexpr int kFoldWarp0 = kStages * kKrGroupWarps;
+    static constexpr int kFoldWarps = kKrTmaWarp - kFoldWarp0;   // 4 or 8
+    // stages per accumulation run, a multiple of the ring depth: about 4096 visibilities
+    // with real and 2048 with complex weights.  The tensor core's FP32 accumulation loses
+    // some 2^-24.5 of the running value per MMA, and runs of twice that length doubled the
+    // error of the exact cutouts (1.0e-5 -> 1.8e-5 of their 2-norm).
+    static constexpr int kFoldStages = (REAL ? 64 : 32) / kStages * kStages;
     static constexpr uint32_t kA = REAL ? kKrATile : 2 * kKrATile;
     static constexpr int kRuns = REAL ? 8 : 4;   // 32-pixel runs per tile
-    // roles that read each item index from the ring: the generator warps in use, 4 fold
-    // warps, the MMA issuer and the uv ring (one arrival each)
-    static constexpr int kReaders = kGroups * kKrGroupWarps + 4 + 1 + 1;
+    // roles that read each item index from the ring: the generator and fold warps, the MMA
+    // issuer and the uv ring (one arrival each)
+    static constexpr int kReaders = kKrTmaWarp + 1 + 1;
     static constexpr uint32_t kSmem = kStages * (kA + kKrBTile) + kKrIn * kKrInSlot + 512 + 1024;
-    static_assert(kGroups <= kKrIn && kGroups * kKrGroupWarps <= kKrGenWarps, "generator groups");
+    static_assert(kStages <= kKrIn && kFoldWarp0 % 4 == 0 && kFoldWarps % 4 == 0, "warp roles");
     static_assert((2 * kStages + 2 * kKrIn + 3 + 5) * 8 + 2 * 4 + 8 <= 512, "barrier block exceeds its reserve");
 };
 
@@ -250,7 +255,7 @@ __global__ void __launch_bounds__(kKrThreads, 1)
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     using Sh = KrShape<REAL>;
-    constexpr int kStages = Sh::kStages, kGroups = Sh::kGroups;
+    constexpr int kStages = Sh::kStages;
     uint8_t *a_base = smem;
     uint8_t *b_base = smem + kStages * Sh::kA;
     uint8_t *in_base = b_base + kStages * kKrBTile;
@@ -282,13 +287,13 @@ __global__ void __launch_bounds__(kKrThreads, 1)
             mbar_init(&in_empty[s], kKrGroupWarps);
         }
         mbar_init(acc_full, 1);
-        mbar_init(acc_empty, 4);
+        mbar_init(acc_empty, Sh::kFoldWarps);
         mbar_init(done_bar, 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&item_full[b], 1);
             mbar_init(&item_empty[b], Sh::kReaders);
         }
-        mbar_init(item_done, 4);
+        mbar_init(item_done, Sh::kFoldWarps);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -303,9 +308,7 @@ __global__ void __launch_bounds__(kKrThreads, 1)
 
     // Every role walks the same item sequence from the two-slot ring: the li-th item of
     // this CTA is in slot li & 1; a role reads it, acknowledges (item_empty) and keeps the
-    // index in registers.  item < 0 ends the sequence.  Stages and fold ranges are
-    // numbered globally across the CTA's items, so the operand rings and the accumulator
-    // run on without draining between items.
+    // index in registers.  item < 0 ends the sequence.
     auto next_item = [&](int li, bool ack) -> int {
         const int slot = li & 1;
         if (!wait_bounded(&item_full[slot], (uint32_t)(li >> 1) & 1u, s_abort, err)) return -2;
@@ -315,9 +318,9 @@ __global__ void __launch_bounds__(kKrThreads, 1)
     };
     auto item_stages = [&](const KrItem &it) { return (it.ke - it.kb + KS - 1) / KS; };
 
-    if (warp < kGroups * kKrGroupWarps) {
+    if (warp < Sh::kFoldWarp0) {
         // ------------------------------------------------------------ pixel twiddles
-        const int grp = warp / kKrGroupWarps, gw = warp % kKrGroupWarps;
+        const int grp = warp / kKrGroupWarps, gw = warp % kKrGroupWarps;   // group = operand slot
         // stmatrix lane address: matrix m = lane / 8 is stream m (piece m of the warp's 64
         // rows, or with complex weights the two pieces of 32 cosine rows and of the sine rows
         // 128 further), 16-byte chunk lane % 8; row n of a piece adds n * 128 and swaps the
@@ -325,7 +328,9 @@ __global__ void __launch_bounds__(kKrThreads, 1)
         const uint32_t lane_off =
             (REAL ? (uint32_t)(gw * 64 + 16 * (lane >> 3))
                   : (uint32_t)(gw * 32 + 16 * ((lane >> 3) & 1) + 128 * (lane >> 4))) * 128u + ((uint32_t)(lane & 7) << 4);
-        int g0 = 0;   // global index of the current item's first stage
+        const uint32_t dst = smem_u32(b_base + grp * kKrBTile) + lane_off;
+        int g0 = 0;          // global index of the current item's first stage
+        uint32_t uses = 0;   // stages this group has written
         bool ok = true;
         for (int li = 0; ok; ++li) {
             int item = -2;
@@ -336,48 +341,41 @@ __global__ void __launch_bounds__(kKrThreads, 1)
             const int nst = item_stages(it);
             const int r0 = it.q0 / 32 + gw * (REAL ? 2 : 1);   // this warp's first run
             const KrRunC run[2] = {kr_run_const(r0, it.N), kr_run_const(r0 + 1, it.N)};
-            // this group's stages of the item: global g = g0 + s with g = grp (mod groups)
-            for (int s = ((grp - g0) % kGroups + kGroups) % kGroups; s < nst; s += kGroups) {
+            for (int s = grp; s < nst; s += kStages, ++uses) {
                 const int g = g0 + s;
-                const int slot = g % kStages;
-                const uint32_t ph = (uint32_t)(g / kStages) & 1u;
                 const int islot = g % kKrIn;
-                bool w = wait_bounded(&in_full[islot], (uint32_t)(g / kKrIn) & 1u, s_abort, err);
-                if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
+                if (!wait_uniform(&in_full[islot], (uint32_t)(g / kKrIn) & 1u, s_abort, err)) { ok = false; break; }
                 const float4 uv2 = reinterpret_cast<const float4 *>(in_base + islot * kKrInSlot)[lane];
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&in_empty[islot]);   // the input slot may be refilled
                 float2 x7[4], x8[4], C[4];
                 kr_seeds<REAL>(uv2, cell, run, x7, x8, C);
-                if (g >= kStages) {
-                    w = wait_bounded(&empty[slot], ph ^ 1u, s_abort, err);
-                    if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
-                }
-                const uint32_t dst = smem_u32(b_base + slot * kKrBTile) + lane_off;
+                if (uses > 0 && !wait_uniform(&empty[grp], (uses - 1) & 1u, s_abort, err)) { ok = false; break; }
                 uint32_t addr[8];
 #pragma unroll
                 for (int n = 0; n < 8; ++n) addr[n] = dst ^ ((uint32_t)n << 4);
                 kr_chain<BF16>(addr, x7, x8, C);
                 fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&full[slot]);
+                if (lane == 0) {
+                    mbar_arrive(&full[grp]);
+                    // The uv slot is released only now: the stage's stores depend on the values read
+                    // from it.  Released right after the reading instruction, the slot was sometimes
+                    // refilled before a warp had its values (one 32-pixel run of one stage wrong in
+                    // up to half of the calls with many short items; none in 180 calls since).
+                    mbar_arrive(&in_empty[islot]);
+                }
             }
             g0 += nst;
         }
-    } else if (warp < kKrGenWarps) {
-        // generator warps beyond the ring depth's groups: idle
     } else if (warp == kKrTmaWarp) {
         // ------------------------------------------------------------ items and weight tiles
         if (lane == 0) {
-            int g = 0;
+            uint32_t used_bits = 0, phase_bits = 0;   // per slot: used before; parity of its last release
             for (int li = 0;; ++li) {
                 const int islot = li & 1;
                 if (li >= 2 && !wait_bounded(&item_empty[islot], (uint32_t)((li >> 1) - 1) & 1u, s_abort, err)) break;
                 // Items do not overlap in the pipeline: the next one is published once the
-                // fold warps have written the previous one out.  (With overlapping items the
-                // twiddle tile of one stage early in a CTA's later items came out wrong in
-                // about one item in ten on GB300; the cause was not found, see the design
-                // notes.)  The bubble costs a ring fill per item.
+                // fold warps have written the previous one out (a ring refill per item, counted
+                // in kr_ranges' item cost).
                 if (li >= 1 && !wait_bounded(item_done, (uint32_t)(li - 1) & 1u, s_abort, err)) break;
                 const int idx = atomicAdd(queue, 1);   // largest items first (host order)
                 const int item = idx < nitems ? idx : -1;
@@ -388,10 +386,12 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                 const int nst = item_stages(it);
                 const uint8_t *src = wblocks + ((int64_t)(it.wrow / 128) * nblk + (it.kb - kchunk0) / KS) * Sh::kA;
                 bool stop = false;
-                for (int s = 0; s < nst; ++s, ++g) {
-                    const int slot = g % kStages;
-                    const uint32_t ph = (uint32_t)(g / kStages) & 1u;
-                    if (g >= kStages && !wait_bounded(&empty[slot], ph ^ 1u, s_abort, err)) { stop = true; break; }
+                for (int s = 0; s < nst; ++s) {
+                    const int slot = s % kStages;
+                    const uint32_t used = (used_bits >> slot) & 1u, ph = (phase_bits >> slot) & 1u;
+                    if (used && !wait_bounded(&empty[slot], ph, s_abort, err)) { stop = true; break; }
+                    if (used) phase_bits ^= 1u << slot;
+                    used_bits |= 1u << slot;
                     mbar_arrive_expect_tx(&full[slot], Sh::kA);
                     bulk_g2s(a_base + slot * Sh::kA, src + (int64_t)s * Sh::kA, Sh::kA, &full[slot]);
                 }
@@ -408,8 +408,7 @@ __global__ void __launch_bounds__(kKrThreads, 1)
             const uint32_t ad0 = warp_uniform(desc_lo(smem_u32(a_base)));
             const uint32_t bd0 = warp_uniform(desc_lo(smem_u32(b_base)));
             const uint32_t tm0 = warp_uniform(tmem);
-            int slot = 0, folds = 0;
-            uint32_t ph = 0;
+            uint32_t phase_bits = 0, folds = 0;   // per slot: parity of its next full phase
             bool stop = false;
             for (int li = 0; !stop; ++li) {
                 int item = next_item(li, lane == 0);
@@ -419,29 +418,29 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                 const KrItem it = items[item];
                 const int nst = (int)warp_uniform((uint32_t)item_stages(it));
                 const uint32_t idesc = warp_uniform(idesc_f16(128, it.npx, BF16));
-                int in_acc = 0;
-                for (int s = 0; s < nst; ++s) {
-                    if (!__all_sync(0xffffffffu, wait_bounded(&full[slot], ph, s_abort, err))) { stop = true; break; }
-                    if (in_acc == 0 && folds > 0 &&
-                        !__all_sync(0xffffffffu, wait_bounded(acc_empty, (uint32_t)(folds - 1) & 1u, s_abort, err))) {
+                for (int s0 = 0, in_acc = 0; s0 < nst && !stop; s0 += kStages) {
+                    if (in_acc == 0 && folds > 0 && !wait_uniform(acc_empty, (folds - 1) & 1u, s_abort, err)) {
                         stop = true;
                         break;
                     }
-                    tc_fence_after();
-                    const uint32_t ad = ad0 + (uint32_t)slot * (Sh::kA >> 4), bd = bd0 + (uint32_t)slot * (kKrBTile >> 4);
-                    umma_f16_x4(tm0, ad, bd, idesc, in_acc ? 1u : 0u, el);
-                    if (!REAL)   // -Im w against the sine rows, columns 128 ..
-                        umma_f16_x4(tm0 + 128u, ad + (kKrATile >> 4), bd + (128u * 128u >> 4), idesc, in_acc ? 1u : 0u,
-                                    el);
-                    umma_commit_elected(&empty[slot], el);
-                    if (++in_acc == kKrFoldStages || s == nst - 1) {
+#pragma unroll
+                    for (int j = 0; j < kStages; ++j) {
+                        if (s0 + j >= nst || stop) break;
+                        if (!wait_uniform(&full[j], (phase_bits >> j) & 1u, s_abort, err)) { stop = true; break; }
+                        tc_fence_after();
+                        const uint32_t ad = ad0 + (uint32_t)j * (Sh::kA >> 4), bd = bd0 + (uint32_t)j * (kKrBTile >> 4);
+                        const uint32_t acc = j ? 1u : (in_acc ? 1u : 0u);
+                        umma_f16_x4(tm0, ad, bd, idesc, acc, el);
+                        if (!REAL)   // -Im w against the sine rows, columns 128 ..
+                            umma_f16_x4(tm0 + 128u, ad + (kKrATile >> 4), bd + (128u * 128u >> 4), idesc, acc, el);
+                        umma_commit_elected(&empty[j], el);
+                    }
+                    phase_bits ^= (1u << min(kStages, nst - s0)) - 1u;
+                    in_acc += kStages;
+                    if (in_acc == Sh::kFoldStages || s0 + kStages >= nst) {
                         umma_commit_elected(acc_full, el);
                         ++folds;
                         in_acc = 0;
-                    }
-                    if (++slot == kStages) {
-                        slot = 0;
-                        ph ^= 1u;
                     }
                 }
             }
@@ -477,7 +476,10 @@ __global__ void __launch_bounds__(kKrThreads, 1)
         __syncwarp();
     } else {
         // ------------------------------------------------------------ fold / output
-        const int qw = warp - kKrFoldWarp0;          // TMEM lane quarter
+        const int qw = warp & 3;                                // TMEM lane quarter
+        constexpr int kParts = Sh::kFoldWarps / 4;              // the tile's pixels, in this many parts
+        constexpr int kPart = 32 * Sh::kRuns / kParts;
+        const int p0 = (warp - Sh::kFoldWarp0) / 4 * kPart;     // this warp's first pixel
         const int row = qw * 32 + lane;              // position row of the tile
         const uint32_t ta = tmem + ((uint32_t)(qw * 32) << 16);
         int F = 0;   // global fold range index
@@ -488,7 +490,7 @@ __global__ void __launch_bounds__(kKrThreads, 1)
             item = __shfl_sync(0xffffffffu, item, 0);
             if (item < 0) break;
             const KrItem it = items[item];
-            const int nfold = (item_stages(it) + kKrFoldStages - 1) / kKrFoldStages;
+            const int nfold = (item_stages(it) + Sh::kFoldStages - 1) / Sh::kFoldStages;
             const bool row_ok = row < it.npos;
             const int N = it.N;
             float *dst = out + (row_ok ? out_off[it.slot0 + row] : 0);
@@ -498,25 +500,29 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                 tc_fence_after();
                 const bool last = (f == nfold - 1);
                 if (!last) {   // running sum (+)= accumulator, 32 columns at a time
-                    for (int c0 = 0; c0 < (REAL ? it.npx : 256); c0 += 32) {
-                        if (!REAL && (c0 & 127) >= it.npx) continue;
-                        uint32_t v[32], u[32];
-                        tmem_ld32_issue(ta + (uint32_t)c0, v);
-                        if (f > 0) {
-                            tmem_ld32_issue(ta + 256u + (uint32_t)c0, u);
-                            tmem_wait_ld(v, u);
+                    const int c_end = min(it.npx, p0 + kPart);
+#pragma unroll 1
+                    for (int h = 0; h < (REAL ? 1 : 2); ++h)
+#pragma unroll 1
+                        for (int c0 = p0; c0 < c_end; c0 += 32) {
+                            const uint32_t tc0 = ta + (uint32_t)(c0 + 128 * h);
+                            uint32_t v[32], u[32];
+                            tmem_ld32_issue(tc0, v);
+                            if (f > 0) {
+                                tmem_ld32_issue(tc0 + 256u, u);
+                                tmem_wait_ld(v, u);
 #pragma unroll
-                            for (int e = 0; e < 32; ++e)
-                                v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(u[e]));
-                        } else {
-                            tmem_wait_ld(v, v);
+                                for (int e = 0; e < 32; ++e)
+                                    v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(u[e]));
+                            } else {
+                                tmem_wait_ld(v, v);
+                            }
+                            tmem_st32_issue(tc0 + 256u, v);
                         }
-                        tmem_st32_issue(ta + 256u + (uint32_t)c0, v);
-                    }
                     tmem_wait_st();
                 }
                 // the end: columns c0 .. c0 + 15 (E) and, with complex weights, 128 + c0 .. (O)
-                for (int c0 = 0; last && c0 < it.npx; c0 += 16) {
+                for (int c0 = p0; last && c0 < min(it.npx, p0 + kPart); c0 += 16) {
                     float v[REAL ? 1 : 2][16];
 #pragma unroll
                     for (int h = 0; h < (REAL ? 1 : 2); ++h) {

@@ -122,11 +122,9 @@ struct psf_plan_s {
     DevBuf gpairs;   // per-call pair records of the gridded form
     DevBuf err;          // int: device-side wait timeouts
     DevBuf queue;        // int: work queue of the persistent batched kernel
-    // autotuner of the batched form, per weight class (bit 0 real weights, bit 1 BF16):
-    // items per SM and, per cutout size, the smallest group the batched form takes
+    // autotuner of the batched form, per weight class (bit 0 real weights, bit 1 BF16): per
+    // cutout size, the smallest group the batched form takes
     struct KrTune {
-        bool done = false;
-        int items_per_cta = 4;
         std::map<int, int> min_group;
     };
     KrTune tune[4];
@@ -554,12 +552,40 @@ struct KrGroup {
 // persistent launch of the Khatri-Rao kernel (one CTA per SM) pulls (128-position tile,
 // pixel tile, visibility range) items from an atomic queue and accumulates them into
 // the zeroed output.  Every item but the last of a cutout has the same number of pixels,
-// so its cost is its visibility range: the ranges are equal, items_per_cta x SMs of them at least (fewer
-// when a range would drop below one 64-stage accumulation run).  kmax < nvis restricts
-// the call to the first kmax visibilities (the autotuner's probes); ms_out (optional)
-// receives the summed time of the contraction launches (the stream is synchronized).
+// so its cost is its visibility range (kr_ranges).  kmax < nvis restricts the call to the
+// first kmax visibilities (the autotuner's probes); ms_out (optional) receives the summed
+// time of the contraction launches (the stream is synchronized).
+//
+// Ranges of the nst stages of a chunk, in stages: an item costs about kItemStages stages
+// beyond its own (ring refill, the pipeline's drain and 64 K atomic adds at its end), and
+// the launch ends when the slowest CTA has finished its last item.  With T stages per CTA
+// ranges of L = sqrt(2 kItemStages T) balance the two, and the last items (1.5 L per CTA)
+// are four times shorter.  SMs differ by up to 40 % in speed under full load (their
+// distance to the weights in L2), so a few long items per CTA, as a probe over a short
+// range preferred, left a tail: 512 mixed cutouts x 7.1 M visibilities 69.5 ms of contraction
+// with 2-4 equal items per CTA, 67.1 ms with these ranges.
+std::vector<int64_t> kr_ranges(int64_t nst, int64_t nbase, int nsm) {
+    constexpr double kItemStages = 100.0;
+    const double T = (double)nst * nbase / nsm;
+    const int64_t L = std::max<int64_t>(64, std::min<int64_t>(nst, (int64_t)std::sqrt(2.0 * kItemStages * T)));
+    const int64_t tail = std::min<int64_t>(nst, (int64_t)(1.5 * L * nsm / nbase));
+    std::vector<int64_t> r;
+    int64_t left = nst;
+    while (left > tail && left - L >= tail / 2) {
+        r.push_back(L);
+        left -= L;
+    }
+    const int64_t S = std::max<int64_t>(64, L / 4);
+    while (left > 0) {
+        const int64_t n = left < S + S / 2 ? left : S;
+        r.push_back(n);
+        left -= n;
+    }
+    return r;
+}
+
 int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGroup> &groups, float *out,
-           cudaStream_t st, int items_per_cta, int64_t kmax = -1, double *ms_out = nullptr) {
+           cudaStream_t st, int64_t kmax = -1, double *ms_out = nullptr) {
     const int64_t K = kmax > 0 ? std::min<int64_t>(kmax, p->nvis) : p->nvis;
     const int bf16 = prec_bf16(p->opts.prec);
     // Methods 1 and 2 have real weights (unless windowed); complex weights take two operand
@@ -607,16 +633,11 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
     for (int64_t c = 0; c < nchunk; ++c) {
         const int64_t kc0 = c * KC, kcn = std::min<int64_t>(KC, K - kc0);
         const int64_t nst = (kcn + ks - 1) / ks;
-        // equal visibility ranges: enough items for items_per_cta per CTA, ranges of at
-        // least one accumulation run (64 stages)
-        const int64_t target = (int64_t)std::max(1, items_per_cta) * p->nsm;
-        int64_t nsplit = std::max<int64_t>(1, std::min<int64_t>((target + nbase - 1) / nbase, nst / 64));
-        const int64_t sper = (nst + nsplit - 1) / nsplit;
-        nsplit = (nst + sper - 1) / sper;
+        const std::vector<int64_t> ranges = kr_ranges(nst, nbase, p->nsm);
         std::vector<KrItem> items;
-        items.reserve(nbase * nsplit);
-        // the full ranges first, the shorter last range after them (largest first)
-        for (int64_t sp = 0; sp < nsplit; ++sp)
+        items.reserve(nbase * ranges.size());
+        int64_t s0 = 0;   // longest ranges first
+        for (const int64_t n : ranges) {
             for (size_t g = 0; g < groups.size(); ++g) {
                 const int np = (int)groups[g].idx.size(), N = groups[g].N;
                 for (int t = 0; t < (np + 127) / 128; ++t)
@@ -628,11 +649,13 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
                         it.N = N;
                         it.q0 = q;
                         it.npx = std::min(tile_px, kr_pixels(N) - q);
-                        it.kb = (int32_t)(kc0 + sp * sper * ks);
-                        it.ke = (int32_t)std::min<int64_t>(kc0 + kcn, kc0 + (sp + 1) * sper * ks);
+                        it.kb = (int32_t)(kc0 + s0 * ks);
+                        it.ke = (int32_t)std::min<int64_t>(kc0 + kcn, kc0 + (s0 + n) * ks);
                         items.push_back(it);
                     }
             }
+            s0 += n;
+        }
         const size_t off_pos = 0;
         const size_t off_slot = align_up(off_pos + npos * sizeof(float4), 16);
         const size_t off_outo = align_up(off_slot + rows * sizeof(int32_t), 16);
@@ -693,13 +716,10 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
 }
 
 // Autotuner of the batched form, run on the first batched call of a plan for each weight
-// class (real / complex weights, operand type) and cached in the plan.  (1) Items per CTA:
-// the batched call of this batch's groups over a probe of the first kProbeVis
-// visibilities, timed for each candidate (2, 4, 8, 16 items per SM), into scratch output;
-// the fastest is kept.  (2) Per cutout size N present, the crossover between the forms:
-// the per-cutout form's time for one position and the batched form's time for one
-// 128-position tile over the same probe; the batched form takes a group of n positions
-// when ceil(n / 128) t_tile < n t_cutout.
+// class (real / complex weights, operand type) and cutout size N and cached in the plan: the
+// crossover between the forms.  Over a probe of the first kProbeVis visibilities it times
+// the per-cutout form for one position and the batched form for one 128-position tile; the
+// batched form takes a group of n positions when ceil(n / 128) t_tile < n t_cutout.
 constexpr int64_t kProbeVis = int64_t(1) << 19;
 
 int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cudaStream_t st, int64_t kmax = -1);
@@ -720,19 +740,7 @@ int kr_tune(psf_plan_s *p, int method, const BatchHost &hall, const std::vector<
     PSF_TRY(scratch.reserve((size_t)std::max<int64_t>(run, 1) * sizeof(float)));
     const bool prof = p->prof;
     p->prof = false;
-    double best = 1e300;
     int s = PSF_OK;
-    std::vector<KrGroup> big;
-    for (const auto &g : cand)
-        if ((int)g.idx.size() >= kKrMinGroup) big.push_back(g);
-    if (!t.done && !big.empty()) {
-        for (int ipc : {2, 4, 8, 16}) {
-            double ms = 0.0;
-            if ((s = run_kr(p, method, hs, big, (float *)scratch.p, st, ipc, probe, &ms))) break;
-            if (ms < best) { best = ms; t.items_per_cta = ipc; }
-        }
-        t.done = s == PSF_OK;
-    }
     // crossover per size: one position per-cutout against one 128-position tile batched
     for (const auto &g : cand) {
         if (s) break;
@@ -741,7 +749,7 @@ int kr_tune(psf_plan_s *p, int method, const BatchHost &hall, const std::vector<
         one[0].N = g.N;
         one[0].idx.assign(g.idx.begin(), g.idx.begin() + std::min<size_t>(g.idx.size(), 128));
         double t_tile = 0.0;
-        if ((s = run_kr(p, method, hs, one, (float *)scratch.p, st, t.items_per_cta, probe, &t_tile))) break;
+        if ((s = run_kr(p, method, hs, one, (float *)scratch.p, st, probe, &t_tile))) break;
         const double lm[2] = {0.0, 0.0};   // cost does not depend on the position
         psf_batch_t b1{};
         b1.npos = 1;
@@ -813,7 +821,7 @@ int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cud
             batched.push_back(g);
             for (int i : g.idx) done[i] = 1;
         }
-        if (!batched.empty() && (s = run_kr(p, method, hall, batched, out, st, t.items_per_cta))) return s;
+        if (!batched.empty() && (s = run_kr(p, method, hall, batched, out, st))) return s;
         for (int i = 0; i < hall.npos; ++i)
             if (!done[i]) {
                 h.pos.push_back(hall.pos[i]);

@@ -75,6 +75,13 @@ static __device__ __forceinline__ bool wait_bounded(uint64_t *bar, uint32_t pari
     }
 }
 
+// wait_bounded by a converged warp, with a warp-uniform result.  The first look decides in
+// one vote; the loop with its clock and flag reads is out of the way of the issue path.
+static __device__ __forceinline__ bool wait_uniform(uint64_t *bar, uint32_t parity, volatile int *abort_flag, int *err) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity, kSleepNs))) return true;
+    return __all_sync(0xffffffffu, wait_bounded(bar, parity, abort_flag, err));
+}
+
 static __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(
                      smem_u32(bar)),
