@@ -101,27 +101,10 @@ __device__ __forceinline__ KrRun kr_run(int r, int N) {
     return KrRun{0, 32 * (r - per_row), 1};
 }
 
-// Nearest integer by adding 1.5 * 2^23 (|x| < 2^22; the conversion unit's rounding
-// instruction runs at a quarter of the FP32 rate).
-__device__ __forceinline__ float nearest(float x) { return __fadd_rn(__fadd_rn(x, 12582912.0f), -12582912.0f); }
-
 __device__ __forceinline__ void cis2(float2 x, float2 &re, float2 &im) {   // exp(2 pi i x) of two phases in turns
     __sincosf(6.28318530717958647f * (x.x - nearest(x.x)), &im.x, &re.x);
     __sincosf(6.28318530717958647f * (x.y - nearest(x.y)), &im.y, &re.y);
 }
-
-// cos and sin of the step 2 pi x from the half angle: the recurrence below amplifies an
-// error of cos(step) by up to the square of its length where the step is small, and
-// 1 - 2 sin^2 (2 cos^2 - 1 beyond a quarter turn) keeps that error at the rounding of 1.
-__device__ __forceinline__ void step1(float x, float &re, float &im) {
-    const float f = x - nearest(x);
-    float s, c;
-    __sincosf(3.14159265358979324f * f, &s, &c);
-    re = fabsf(f) < 0.25f ? fmaf(-2.0f * s, s, 1.0f) : fmaf(2.0f * c, c, -1.0f);
-    im = 2.0f * s * c;
-}
-
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
 // (ar + i ai)(br + i bi) for two visibilities at a time; nbi = -bi.
 __device__ __forceinline__ float2 mul_re(float2 ar, float2 ai, float2 br, float2 nbi) {
@@ -137,8 +120,8 @@ struct KrSteps {
 };
 __device__ __forceinline__ KrSteps kr_steps(float2 th) {
     KrSteps S;
-    step1(th.x, S.sr.x, S.si.x);
-    step1(th.y, S.sr.y, S.si.y);
+    step_phasor(th.x, S.sr.x, S.si.x);
+    step_phasor(th.y, S.sr.y, S.si.y);
     const float2 f = make_float2(th.x - nearest(th.x), th.y - nearest(th.y));
     cis2(make_float2(16.0f * f.x, 16.0f * f.y), S.tr, S.ti);
     return S;
@@ -148,16 +131,14 @@ template <int BF16, int ROW>
 __device__ __forceinline__ void kr_row(const uint32_t (&addr)[8], const float2 (&x)[4]) {
     const uint32_t v0 = pack2<BF16>(x[0].x, x[0].y), v1 = pack2<BF16>(x[1].x, x[1].y);
     const uint32_t v2 = pack2<BF16>(x[2].x, x[2].y), v3 = pack2<BF16>(x[3].x, x[3].y);
-    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0 + %5], {%1, %2, %3, %4};" ::"r"(addr[ROW & 7]), "r"(v0),
-                 "r"(v1), "r"(v2), "r"(v3), "n"(ROW * 128)
-                 : "memory");
+    stmatrix_x4_at<ROW * 128>(addr[ROW & 7], v0, v1, v2, v3);
 }
 
 // Rows 0 .. 15 of four 16-pixel pieces (one stream per stmatrix matrix), from their rows 7
 // and 8 outwards: x_{n+1} = C x_n - x_{n-1}, C = 2 cos(step), one packed FMA per pixel and
 // two visibilities (a complex step takes four), at most eight steps from a seed, so that
 // rounding grows by less than ten.  The subtraction is left to the output: the rows are
-// carried as y = +-x with the signs + - - + + - - + ... (kr_sign), for which every step is
+// carried as y = +-x with the signs + - - + + - - + ... (row_sign), for which every step is
 // y = (+-C) y + y.
 template <int BF16>
 __device__ __forceinline__ void kr_chain(const uint32_t (&addr)[8], const float2 (&x7)[4], const float2 (&x8)[4],
@@ -201,9 +182,6 @@ __device__ __forceinline__ void kr_chain(const uint32_t (&addr)[8], const float2
     kr_row<BF16, 15>(addr, fc);
     kr_row<BF16, 0>(addr, bc);
 }
-
-// Sign with which kr_chain carries pixel c of a tile.
-__device__ __forceinline__ constexpr float kr_sign(int c) { return ((c + 1) & 2) ? -1.0f : 1.0f; }
 
 // A run's constants: the phase of its row 7 is tu cu + tv cv (turns), its step tu or tv.
 struct KrRunC {
@@ -546,7 +524,7 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                     const bool mirrored = !run.along_m && run.j0 > N / 2;
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
-                        const float E = kr_sign(e) * v[0][e], O = REAL ? 0.f : kr_sign(e) * v[REAL ? 0 : 1][e];
+                        const float E = row_sign(e) * v[0][e], O = REAL ? 0.f : row_sign(e) * v[REAL ? 0 : 1][e];
                         const int j = run.j0 + t0 + e;
                         if (!run.along_m || (j >= 1 && j < N / 2)) atomicAdd(dst + pix + e * pstep, E + O);
                         if (mirrored && run.i0 + t0 + e >= 1) atomicAdd(dst + N * N + N - pix - e, E - O);

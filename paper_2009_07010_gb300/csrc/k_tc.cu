@@ -7,21 +7,11 @@
 //   A'[j][2k] = Re c, A'[j][2k+1] = Im c,  B'[i][2k] = Re a, B'[i][2k+1] = -Im a,
 //   P = A' B'^T  with K' = 2K (FP16 or BF16 operands, FP32 accumulation in TMEM).
 //
-// Warp roles (736 threads):
-//   warps 0-15  operand generators (four groups on stages s mod 4, two chains per warp
-//               and stage): per pipeline stage of 32 visibilities each lane
-//               owns one visibility and walks a 32-row recurrence chain
-//               (seed and step from the MUFU sin/cos of the reduced phase, then
-//               complex multiplication), writing FP16/BF16 pairs straight into the
+// Warp roles (TcShape; numbers for the 16 generator warps of most instances):
+//   warps 0-15  operand generators (groups on stages s mod groups): per pipeline stage of
+//               32 visibilities each lane owns one visibility and generates 32 or 64
+//               twiddle rows (tw_rows), writing FP16/BF16 pairs straight into the
 //               128-byte-swizzled K-major shared-memory layout the MMA reads;
-//   warps 20, 22  TMEM allocation and the tcgen05.mma issue: with NISS = 2 (tiles of at
-//               most 128 columns) warp 20 issues the even stages and warp 22 the odd
-//               ones, each into accumulators of its own, so that one issuer's barrier
-//               wait (an mbarrier round trip during which a lone issuer leaves the
-//               tensor core idle) overlaps the other issuer's MMAs; with NISS = 1
-//               warp 20 issues every stage;
-//   warp 21     the uv/w input ring: one bulk copy pair per stage, refilled when the
-//               generator group of the stage has read it (`in_empty`);
 //   warps 16-19 drain: every kDrainStages stages the issuers switch to their second
 //               TMEM accumulator while these warps read the first ones (tcgen05.ld),
 //               add them and add the sum into the CTA's FP32 partial tile in global
@@ -30,12 +20,18 @@
 //               error-free TwoSum whose rounding error goes back into the drained
 //               accumulator, on which the issuer's next range in that buffer
 //               accumulates (compensated summation, the correction carried by the
-//               tensor core).
+//               tensor core);
+//   warps 20, 22  TMEM allocation and the tcgen05.mma issue: with NISS = 2 (tiles of at
+//               most 128 columns) one issues the even stages and one the odd ones, each
+//               into accumulators of its own, so that one issuer's barrier wait overlaps
+//               the other issuer's MMAs; with NISS = 1 one issues every stage;
+//   warp 21     the uv/w input ring: one bulk copy pair per stage, refilled when the
+//               generator group of the stage has written it (`in_empty`).
 // Stages are handed over with mbarriers (input copies -> generators: `in_full`,
 // generators -> input warp: `in_empty`, generators -> MMA: `full`, MMA commit ->
 // generators: `empty`, MMA commit -> drain: `acc_full`, drain -> MMA: `acc_empty`).
-// An issuing thread does nothing per stage but wait, issue and commit: MMA issue
-// blocks the thread, so its serial latency bounds the stage rate.  Every wait is bounded by a wall-clock limit; on
+// An issuing warp does nothing per stage but wait, issue and commit: MMA issue blocks it,
+// so its serial latency bounds the stage rate.  Every wait is bounded by a wall-clock limit; on
 // expiry the CTA raises the plan's error flag, stops all roles, waits (bounded) for
 // its bulk copies and issued MMAs and frees TMEM.
 #include <cuda_bf16.h>
@@ -50,20 +46,38 @@ using namespace tc;
 
 constexpr int kInStages = 16;      // per-visibility input (uv, w) ring depth
 constexpr int kKS = 32;            // complex visibilities per stage (K' = 64 = one 128 B row)
-constexpr int kGenWarps = 16;      // four groups of 4; group g generates stages s = g (mod 4)
-constexpr int kGroupWarps = 4;
-constexpr int kGroups = kGenWarps / kGroupWarps;
-// A group waiting for slot reuse (stage s - S consumed) must find the slot's previous
-// phase (stage s - 2S) already consumed, or the parity test of the barrier aliases;
-// that holds when the group's previous stage s - kGroups waited for stage
-// s - kGroups - S >= s - 2S, i.e. kGroups <= S for every ring depth S used (4, 6, 8).
-static_assert(kGroups <= 4, "generator groups must not exceed the smallest operand ring depth");
-static_assert(kGroups <= kInStages, "generator groups must not exceed the input ring depth");
-constexpr int kDrainWarp0 = 16;
-constexpr int kMmaWarp = 20;
-constexpr int kInWarp = 21;
-constexpr int kMma2Warp = 22;
-constexpr int kThreads = 23 * 32;
+// Warp roles of an instance.  Group g of the generator warps writes the stages s = g (mod
+// groups).  A group waiting for slot reuse (stage s - S consumed) must find the slot's
+// previous phase (stage s - 2S) already consumed, or the parity test of the barrier aliases;
+// that holds when the group's previous stage s - groups waited for stage s - groups - S >=
+// s - 2S, i.e. groups <= S.  With two issuers the group count must also be even: each issuer
+// commits in order, but the two do not order each other, so both stages have to belong to
+// the same issuer (an instance with five groups aliased and gave up its bounded waits).
+//
+// The generators bound the kernel (4 h MeerKAT cutout, exact: 3.72 ms without the MMAs, 2.50 ms
+// without the twiddle rows, 3.78 ms together, before the last two of the following).  Seeds,
+// barrier waits and loop code are about 130 of a warp's 290-350 instructions per stage, so
+// the instances of the 128-pixel cutout give a warp 64 rows: with complex weights two warps
+// take A, two the conjugate-symmetric B, the roles rotating with the group so that each
+// falls on every scheduler (warp mod 4); in the fused form one takes A and two take B, one
+// per weight.  Exact 4.39 -> 3.56 ms, fused 5.95 -> 4.60 ms.  24 warps of 64 registers were
+// slower (recomputed addresses: 312 M -> 395 M instructions; fused 5.6 ms), as were six
+// groups of two (3.85 ms) or three warps (3.69 ms) for the exact form.
+template <int kStages, int NISS, int MIR, int SPLIT>
+struct TcShape {
+    static constexpr bool kTall = !SPLIT && ((MIR == 0 && kStages == 6) || (MIR == 4 && kStages == 4));
+    static constexpr int kGroupWarps = kTall && MIR == 4 ? 3 : 4;
+    static constexpr int kGroups0 = kStages < 4 ? kStages : 4;
+    static constexpr int kGroups = NISS == 2 ? (kGroups0 & ~1) : kGroups0;
+    static constexpr int kGen = kGroups * kGroupWarps;
+    static constexpr int kDrainWarp0 = (kGen + 3) / 4 * 4;   // lane quarter = warp mod 4
+    static constexpr int kMmaWarp = kDrainWarp0 + 4;
+    static constexpr int kInWarp = kMmaWarp + 1;
+    static constexpr int kMma2Warp = kMmaWarp + 2;
+    static constexpr int kThreads = (kMmaWarp + 3) * 32;
+    static_assert(NISS == 1 || kGroups % 2 == 0, "two issuers need an even number of generator groups");
+    static_assert(kGroups <= kStages && kGroups <= kInStages, "generator groups exceed a ring depth");
+};
 constexpr int kDrainStages = 64;   // stages accumulated in TMEM between drains
 // Split precision: the tensor core's FP32 accumulation loses about 2^-24.5 of the running
 // value per added MMA (measured: the error of a cutout grows with the MMAs accumulated
@@ -84,215 +98,126 @@ __device__ __forceinline__ void two_sum(float a, float b, float &t, float &e) {
     const float bp = t - a;
     e = (a - (t - bp)) + (b - bp);
 }
+// *p += v without reading the old value back.
+__device__ __forceinline__ void red_add(float *p, float v) {
+    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
 constexpr int kATileBytes = 128 * 128;
-// One 32-row twiddle chain of one visibility (this lane), rows r = 0..31 of `base`:
-// value(r) = [w] exp(2 pi i theta (n0 + r)), written as an FP16/BF16 (re, im) pair at
-// the lane's K-major swizzled slot.  The chain runs as eight interleaved 4-row pieces
-// (seeds at r = 0, 4, ..., 28) held in four packed FP32x2 pairs, so each step is four
-// independent packed complex multiplications, and the eight rows of a step leave in
-// two stmatrix.
-// MIRROR: the chain also writes the complex conjugate of row r at row R0 - r (mbase =
-// tile + R0 * 128 with R0 a multiple of 8; the packed pair's imaginary half is the
-// high 16 bits, so conjugation is a sign-bit XOR), and with `tail` the conjugate of
-// the value one step past the last row at `tail_addr` (row 0 of the tile).
-// CPLX: each row value z is also written as (-Im z, Re z) at row r of base + mbase
-// (the second half of a doubled B tile: with z = conj(a) these rows give the
-// imaginary part of the contraction).
-// SPLIT: every value is also written as its low part (value - rounded value, rounded
-// to 16 bits) at the same position lo_off bytes further on (the lo tile of a split
-// precision stage); conjugation of the low part is the same sign-bit XOR.
-// The step exp(2 pi i theta) of a chain and its 4-, 8- and 16-row strides (squarings):
-// shared by the chains of one visibility that have the same theta.
-struct ChainSteps {
-    float2 st, s4, s8, s16;
+// Twiddle rows of one visibility (this lane): value(r) = [w] exp(2 pi i theta (n0 + r)),
+// written as an FP16/BF16 (re, im) pair at the lane's K-major swizzled slot, four rows (one
+// of each of four pieces of PIECE = 8 or 16 rows) per stmatrix.  Each piece is seeded at its
+// two middle rows and runs outwards by x_{n+1} = C x_n - x_{n-1}, C = 2 cos(step): one packed
+// FMA per row, where the complex step of a phasor recurrence takes two (and its seeds every
+// fourth row more): 888 M warp instructions of the exact launch on the 1 h MeerKAT cutout
+// became 638 M.  The subtraction is left to the output: the rows are carried with the signs
+// of row_sign, for which every step is y = (+-C) y + y.
+// Seeds: sine/cosine evaluations for the middle row of the first piece, the step and the
+// stride between pieces; three squarings and products give the rest.
+struct TwSeeds {
+    float2 xa[4], xb[4];   // rows PIECE/2 - 1 and PIECE/2 of the four pieces
+    float2 C;              // (2 cos(step), 2 cos(step))
 };
-__device__ __forceinline__ ChainSteps chain_steps(float theta) {
-    ChainSteps S;
-    S.st = cis_turns(theta);
-    const float2 s2 = cmulf(S.st, S.st);
-    S.s4 = cmulf(s2, s2);
-    S.s8 = cmulf(S.s4, S.s4);
-    S.s16 = cmulf(S.s8, S.s8);
+
+template <int PIECE>
+__device__ __forceinline__ TwSeeds tw_seeds(float theta, int n0, float2 wk, bool weighted) {
+    TwSeeds S;
+    float2 st;
+    step_phasor(theta, st.x, st.y);
+    const float f = theta - nearest(theta);
+    const float2 s1 = cis_fast((float)PIECE * f), s2 = cmulf(s1, s1);
+    float2 z = cis_fast(theta * (float)(n0 + PIECE / 2 - 1));
+    if (weighted) z = cmulf(z, wk);
+    S.xa[0] = z;
+    S.xa[1] = cmulf(z, s1);
+    S.xa[2] = cmulf(z, s2);
+    S.xa[3] = cmulf(S.xa[1], s2);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) S.xb[m] = cmulf(S.xa[m], st);
+    S.C = make_float2(2.0f * st.x, 2.0f * st.x);
     return S;
 }
 
-template <int BF16, bool MIRROR = false, bool CPLX = false, bool SPLIT = false>
-__device__ __forceinline__ void gen_chain32_s(const ChainSteps &S, uint32_t base, const uint32_t (&off)[8],
-                                              float theta, int n0, float2 wk, bool weighted, uint32_t mbase = 0,
-                                              bool tail = false, uint32_t tail_addr = 0, uint32_t lo_off = 0) {
-    // eight interleaved 4-row pieces: rows q + 4p (p = 0..7) at step q = 0..3.  Two
-    // sine/cosine evaluations per chain (row 0 and the step, the latter in S); the piece
-    // seeds follow by complex multiplication with the 4- and 16-row strides (squarings
-    // of the step), which keeps the MUFU pipe to 4 instructions per 32 rows.
-    const float2 st = S.st, s4 = S.s4, s8 = S.s8, s16 = S.s16;
-    float2 z[8];
-    z[0] = cis_turns(theta * (float)n0);
-    if (weighted) z[0] = cmulf(z[0], wk);
-    z[1] = cmulf(z[0], s4);
-    z[2] = cmulf(z[0], s8);
-    z[3] = cmulf(z[1], s8);
+// Store of one row of each piece.  at: the lane's address of row 0 (piece lane / 8, chunk
+// lane % 8 of its tile); MIRROR: the conjugates (a sign-bit XOR of the imaginary half) go to
+// the rows R0 - r, mat being the lane's address of row R0; CPLX: (-Im z, Re z) at the same rows
+// cplx_off bytes further on; SPLIT: the low parts (value minus its rounding, rounded again)
+// lo_off bytes further on.
+template <int BF16, int ROW, bool MIRROR, bool CPLX, bool SPLIT>
+__device__ __forceinline__ void tw_row(uint32_t at, uint32_t mat, uint32_t cplx_off, uint32_t lo_off,
+                                       const float2 (&x)[4]) {
+    constexpr uint32_t kConj = 0x80000000u;
+    constexpr uint32_t kSw = (uint32_t)(ROW & 7) << 4, kMsw = (uint32_t)((8 - (ROW & 7)) & 7) << 4;
+    uint32_t v[4];
 #pragma unroll
-    for (int pc = 4; pc < 8; ++pc) z[pc] = cmulf(z[pc - 4], s16);
-    // packed pairs: P0 = rows (q, q+16), P1 = (q+8, q+24), P2 = (q+4, q+20), P3 = (q+12, q+28)
-    float2 re[4], im[4];
-    re[0] = make_float2(z[0].x, z[4].x); im[0] = make_float2(z[0].y, z[4].y);
-    re[1] = make_float2(z[2].x, z[6].x); im[1] = make_float2(z[2].y, z[6].y);
-    re[2] = make_float2(z[1].x, z[5].x); im[2] = make_float2(z[1].y, z[5].y);
-    re[3] = make_float2(z[3].x, z[7].x); im[3] = make_float2(z[3].y, z[7].y);
-    const float2 sr = make_float2(st.x, st.x), si = make_float2(st.y, st.y), nsi = make_float2(-st.y, -st.y);
+    for (int m = 0; m < 4; ++m) v[m] = pack2<BF16>(x[m].x, x[m].y);
+    const uint32_t addr = at ^ kSw, maddr = mat ^ kMsw;
+    stmatrix_x4_at<ROW * 128>(addr, v[0], v[1], v[2], v[3]);
+    if (MIRROR) stmatrix_x4_at<-ROW * 128>(maddr, v[0] ^ kConj, v[1] ^ kConj, v[2] ^ kConj, v[3] ^ kConj);
+    if (CPLX)
+        stmatrix_x4_at<ROW * 128>(addr + cplx_off, pack2<BF16>(-x[0].y, x[0].x), pack2<BF16>(-x[1].y, x[1].x),
+                                  pack2<BF16>(-x[2].y, x[2].x), pack2<BF16>(-x[3].y, x[3].x));
+    if (SPLIT) {
+        uint32_t l[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        // rows q, q+8, q+16, q+24 and rows q+4, q+12, q+20, q+28
-        // matrix m of a mirrored store at offset q' writes row R0 - (q' + 8 m), chunk
-        // (lane mod 8) swizzled with (-q') mod 8
-        constexpr uint32_t kConj = 0x80000000u;
-        const uint32_t ln = threadIdx.x & 31u, ca = ln & 7u;
-        {
-            const uint32_t v0 = pack2<BF16>(re[0].x, im[0].x), v1 = pack2<BF16>(re[1].x, im[1].x);
-            const uint32_t v2 = pack2<BF16>(re[0].y, im[0].y), v3 = pack2<BF16>(re[1].y, im[1].y);
-            // without mirroring the row addresses are recomputed from the lane (cheaper than
-            // holding eight offsets at this kernel's register budget)
-            const uint32_t addr = MIRROR ? base + off[q]
-                                         : base + (((threadIdx.x >> 3) & 3u) << 10) + (uint32_t)q * 128u +
-                                               (((threadIdx.x & 7u) ^ (uint32_t)q) << 4);
-            stmatrix_x4(addr, v0, v1, v2, v3);
-            uint32_t l0 = 0u, l1 = 0u, l2 = 0u, l3 = 0u;
-            if (SPLIT) {
-                l0 = pack2_lo<BF16>(re[0].x, im[0].x, v0);
-                l1 = pack2_lo<BF16>(re[1].x, im[1].x, v1);
-                l2 = pack2_lo<BF16>(re[0].y, im[0].y, v2);
-                l3 = pack2_lo<BF16>(re[1].y, im[1].y, v3);
-                stmatrix_x4(addr + lo_off, l0, l1, l2, l3);
-            }
-            if (MIRROR) {
-                const uint32_t maddr = mbase - (ln >> 3) * 1024u - (uint32_t)q * 128u + ((ca ^ ((8u - q) & 7u)) << 4);
-                stmatrix_x4(maddr, v0 ^ kConj, v1 ^ kConj, v2 ^ kConj, v3 ^ kConj);
-                if (SPLIT) stmatrix_x4(maddr + lo_off, l0 ^ kConj, l1 ^ kConj, l2 ^ kConj, l3 ^ kConj);
-            }
-            if (CPLX)
-                stmatrix_x4(base + mbase + (((threadIdx.x >> 3) & 3u) << 10) + (uint32_t)q * 128u +
-                                (((threadIdx.x & 7u) ^ (uint32_t)q) << 4),
-                            pack2<BF16>(-im[0].x, re[0].x), pack2<BF16>(-im[1].x, re[1].x),
-                            pack2<BF16>(-im[0].y, re[0].y), pack2<BF16>(-im[1].y, re[1].y));
-        }
-        {
-            const uint32_t v4 = pack2<BF16>(re[2].x, im[2].x), v5 = pack2<BF16>(re[3].x, im[3].x);
-            const uint32_t v6 = pack2<BF16>(re[2].y, im[2].y), v7 = pack2<BF16>(re[3].y, im[3].y);
-            const uint32_t addr = MIRROR ? base + off[q + 4]
-                                         : base + (((threadIdx.x >> 3) & 3u) << 10) + (uint32_t)(q + 4) * 128u +
-                                               (((threadIdx.x & 7u) ^ (uint32_t)(q + 4)) << 4);
-            stmatrix_x4(addr, v4, v5, v6, v7);
-            uint32_t l4 = 0u, l5 = 0u, l6 = 0u, l7 = 0u;
-            if (SPLIT) {
-                l4 = pack2_lo<BF16>(re[2].x, im[2].x, v4);
-                l5 = pack2_lo<BF16>(re[3].x, im[3].x, v5);
-                l6 = pack2_lo<BF16>(re[2].y, im[2].y, v6);
-                l7 = pack2_lo<BF16>(re[3].y, im[3].y, v7);
-                stmatrix_x4(addr + lo_off, l4, l5, l6, l7);
-            }
-            if (MIRROR) {
-                const uint32_t maddr =
-                    mbase - (ln >> 3) * 1024u - (uint32_t)(q + 4) * 128u + ((ca ^ ((4u - q) & 7u)) << 4);
-                stmatrix_x4(maddr, v4 ^ kConj, v5 ^ kConj, v6 ^ kConj, v7 ^ kConj);
-                if (SPLIT) stmatrix_x4(maddr + lo_off, l4 ^ kConj, l5 ^ kConj, l6 ^ kConj, l7 ^ kConj);
-            }
-            if (CPLX)
-                stmatrix_x4(base + mbase + (((threadIdx.x >> 3) & 3u) << 10) + (uint32_t)(q + 4) * 128u +
-                                (((threadIdx.x & 7u) ^ (uint32_t)(q + 4)) << 4),
-                            pack2<BF16>(-im[2].x, re[2].x), pack2<BF16>(-im[3].x, re[3].x),
-                            pack2<BF16>(-im[2].y, re[2].y), pack2<BF16>(-im[3].y, re[3].y));
-        }
-        if (q < 3) {
-#pragma unroll
-            for (int pp = 0; pp < 4; ++pp) {
-                const float2 t = __fmul2_rn(im[pp], nsi), u = __fmul2_rn(im[pp], sr);
-                im[pp] = __ffma2_rn(re[pp], si, u);
-                re[pp] = __ffma2_rn(re[pp], sr, t);
-            }
-        }
+        for (int m = 0; m < 4; ++m) l[m] = pack2_lo<BF16>(x[m].x, x[m].y, v[m]);
+        stmatrix_x4_at<ROW * 128>(addr + lo_off, l[0], l[1], l[2], l[3]);
+        if (MIRROR)
+            stmatrix_x4_at<-ROW * 128>(maddr + lo_off, l[0] ^ kConj, l[1] ^ kConj, l[2] ^ kConj, l[3] ^ kConj);
     }
-    if (MIRROR && tail) {   // row 32 = piece 7 (row 31, the .y half of pair 3) one step on
-        const float r32 = re[3].y * st.x - im[3].y * st.y, i32 = re[3].y * st.y + im[3].y * st.x;
+}
+
+// The 4 PIECE rows from the tile row at `base` (a multiple of 8 rows).  MIRROR:
+// conjugates at the rows R0 - r, mbase = the address of row R0 (a multiple of 8); with
+// `tail` the conjugate of the value one step past the last row at `tail_addr` (row 0).
+template <int BF16, int PIECE, bool MIRROR = false, bool CPLX = false, bool SPLIT = false>
+__device__ __forceinline__ void tw_rows(const TwSeeds &S, uint32_t base, uint32_t mbase = 0, bool tail = false,
+                                        uint32_t tail_addr = 0, uint32_t cplx_off = 0, uint32_t lo_off = 0) {
+    static_assert(PIECE == 8 || PIECE == 16, "piece");
+    const uint32_t piece = (threadIdx.x >> 3) & 3u, chunk = (threadIdx.x & 7u) << 4;
+    const uint32_t at = base + piece * (PIECE * 128u) + chunk, mat = mbase - piece * (PIECE * 128u) + chunk;
+    const float2 nC = neg2(S.C);
+    float2 fp[4], fc[4], bp[4], bc[4];
+#define TW_ROW(R, X) tw_row<BF16, R, MIRROR, CPLX, SPLIT>(at, mat, cplx_off, lo_off, X)
+    TW_ROW(PIECE / 2 - 1, S.xa);
+    TW_ROW(PIECE / 2, S.xb);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        fp[m] = bc[m] = S.xa[m];
+        fc[m] = bp[m] = S.xb[m];
+    }
+#define TW_STEP(K)                                                                      \
+    {                                                                                   \
+        _Pragma("unroll") for (int m = 0; m < 4; ++m) {                                 \
+            const float2 c = ((K) & 1) ? nC : S.C;                                      \
+            const float2 f = __ffma2_rn(c, fc[m], fp[m]), b = __ffma2_rn(c, bc[m], bp[m]); \
+            fp[m] = fc[m];                                                              \
+            fc[m] = f;                                                                  \
+            bp[m] = bc[m];                                                              \
+            bc[m] = b;                                                                  \
+        }                                                                               \
+        TW_ROW(PIECE / 2 + (K), fc);                                                    \
+        TW_ROW(PIECE / 2 - 1 - (K), bc);                                                \
+    }
+    TW_STEP(1)
+    TW_STEP(2)
+    TW_STEP(3)
+    if constexpr (PIECE == 16) {
+        TW_STEP(4)
+        TW_STEP(5)
+        TW_STEP(6)
+        TW_STEP(7)
+    }
+#undef TW_STEP
+#undef TW_ROW
+    if (MIRROR && tail) {   // row 4 PIECE: one more step of the last piece (sign +)
+        const float2 x = __ffma2_rn(S.C, fc[3], fp[3]);
         const uint32_t lane = threadIdx.x & 31u;
-        // row 0: chunk lane / 4 (unswizzled), pair lane mod 4
-        const uint32_t h = pack2<BF16>(r32, -i32);
+        const uint32_t h = pack2<BF16>(x.x, -x.y);   // row 0: chunk lane / 4 (unswizzled), pair lane mod 4
         asm volatile("st.shared.b32 [%0], %1;" ::"r"(tail_addr + lane * 4u), "r"(h) : "memory");
         if (SPLIT)
             asm volatile("st.shared.b32 [%0], %1;" ::"r"(tail_addr + lo_off + lane * 4u),
-                         "r"(pack2_lo<BF16>(r32, -i32, h))
+                         "r"(pack2_lo<BF16>(x.x, -x.y, h))
                          : "memory");
-    }
-}
-
-template <int BF16, bool MIRROR = false, bool CPLX = false, bool SPLIT = false>
-__device__ __forceinline__ void gen_chain32(uint32_t base, const uint32_t (&off)[8], float theta, int n0, float2 wk,
-                                            bool weighted, uint32_t mbase = 0, bool tail = false,
-                                            uint32_t tail_addr = 0, uint32_t lo_off = 0) {
-    gen_chain32_s<BF16, MIRROR, CPLX, SPLIT>(chain_steps(theta), base, off, theta, n0, wk, weighted, mbase, tail,
-                                             tail_addr, lo_off);
-}
-
-// Two real-weight copies of one conjugate-symmetric 32-row chain of unweighted twiddles
-// (the fused uv + image-plane form): the value z(r) of row R0 + r is stored as
-// (wa z) at base + r rows and (wb z) at base + half_off + r rows, each with its
-// conjugate at the mirrored row R0 - r (mbase, mbase + half_off); with `tail` the
-// conjugates of (wa, wb) x the value one step past the last row go to row 0 of each
-// half (tail_addr, tail_addr + half_off).
-template <int BF16>
-__device__ __forceinline__ void gen_chain32_dual(uint32_t base, uint32_t mbase, uint32_t half_off, float theta,
-                                                 int n0, float wa, float wb, bool tail, uint32_t tail_addr) {
-    const float2 st = cis_turns(theta);
-    float2 z[8];
-    z[0] = cis_turns(theta * (float)n0);
-    const float2 s2 = cmulf(st, st), s4 = cmulf(s2, s2), s8 = cmulf(s4, s4), s16 = cmulf(s8, s8);
-    z[1] = cmulf(z[0], s4);
-    z[2] = cmulf(z[0], s8);
-    z[3] = cmulf(z[1], s8);
-#pragma unroll
-    for (int pc = 4; pc < 8; ++pc) z[pc] = cmulf(z[pc - 4], s16);
-    float2 re[4], im[4];
-    re[0] = make_float2(z[0].x, z[4].x); im[0] = make_float2(z[0].y, z[4].y);
-    re[1] = make_float2(z[2].x, z[6].x); im[1] = make_float2(z[2].y, z[6].y);
-    re[2] = make_float2(z[1].x, z[5].x); im[2] = make_float2(z[1].y, z[5].y);
-    re[3] = make_float2(z[3].x, z[7].x); im[3] = make_float2(z[3].y, z[7].y);
-    const float2 sr = make_float2(st.x, st.x), si = make_float2(st.y, st.y), nsi = make_float2(-st.y, -st.y);
-    constexpr uint32_t kConj = 0x80000000u;
-    const uint32_t ln = threadIdx.x & 31u, ca = ln & 7u;
-    const uint32_t lrow = (((threadIdx.x >> 3) & 3u) << 10);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float2 wv = h ? make_float2(wb, wb) : make_float2(wa, wa);
-            const uint32_t ho = h ? half_off : 0u;
-#pragma unroll
-            for (int m = 0; m < 2; ++m) {   // matrices of rows q + 8 m' (m = 0) and q + 4 + 8 m' (m = 1)
-                const float2 ra = __fmul2_rn(re[2 * m], wv), ia = __fmul2_rn(im[2 * m], wv);
-                const float2 rb = __fmul2_rn(re[2 * m + 1], wv), ib = __fmul2_rn(im[2 * m + 1], wv);
-                const uint32_t v0 = pack2<BF16>(ra.x, ia.x), v1 = pack2<BF16>(rb.x, ib.x);
-                const uint32_t v2 = pack2<BF16>(ra.y, ia.y), v3 = pack2<BF16>(rb.y, ib.y);
-                const uint32_t qq = (uint32_t)(q + 4 * m);
-                stmatrix_x4(base + ho + lrow + qq * 128u + ((ca ^ qq) << 4), v0, v1, v2, v3);
-                stmatrix_x4(mbase + ho - lrow - qq * 128u + ((ca ^ ((8u - qq) & 7u)) << 4), v0 ^ kConj, v1 ^ kConj,
-                            v2 ^ kConj, v3 ^ kConj);
-            }
-        }
-        if (q < 3) {
-#pragma unroll
-            for (int pp = 0; pp < 4; ++pp) {
-                const float2 t = __fmul2_rn(im[pp], nsi), u = __fmul2_rn(im[pp], sr);
-                im[pp] = __ffma2_rn(re[pp], si, u);
-                re[pp] = __ffma2_rn(re[pp], sr, t);
-            }
-        }
-    }
-    if (tail) {   // row 32 = piece 7 (row 31, the .y half of pair 3) one step on
-        const float r32 = re[3].y * st.x - im[3].y * st.y, i32 = re[3].y * st.y + im[3].y * st.x;
-        asm volatile("st.shared.b32 [%0], %1;" ::"r"(tail_addr + ln * 4u), "r"(pack2<BF16>(wa * r32, -wa * i32))
-                     : "memory");
-        asm volatile("st.shared.b32 [%0], %1;" ::"r"(tail_addr + half_off + ln * 4u),
-                     "r"(pack2<BF16>(wb * r32, -wb * i32))
-                     : "memory");
     }
 }
 
@@ -339,8 +264,14 @@ __host__ __device__ inline SmemLayout smem_layout(int ncols_max, int kStages, ui
 // each stage issues A_hi B_hi + A_hi B_lo + A_lo B_hi into the same accumulator (the
 // lo x lo term is below the 16-bit rounding of the lo parts).  The stages are twice as
 // large, so the ring holds 3 or 4 of them and as many generator groups run.
+template <int MIR>
+__device__ __forceinline__ bool whole_cutout(const TcItem &it) {   // conjugate-symmetric generation
+    return MIR == 2 || MIR == 4 ||
+           (MIR == 1 && it.j0 == 0 && it.i0 == 0 && it.ncols == it.N && it.N <= 128 && (it.N & 63) == 0);
+}
+
 template <int BF16, int kStages, int NISS, int MIR, int SPLIT = 0>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(TcShape<kStages, NISS, MIR, SPLIT>::kThreads, 1)
     k_psf_tc(const float2 *__restrict__ uv, const float2 *__restrict__ w, int64_t ldw,
              const TcItem *__restrict__ items, int ncols_max, float cell, float *__restrict__ partial,
              int64_t split_stride, int *err, const float2 *__restrict__ w2, int64_t part2) {
@@ -349,16 +280,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     constexpr int kBMul = (MIR == 4 || MIR == 5) ? 2 : 1;           // B rows per output column
     constexpr uint32_t kSlot = (MIR == 4) ? kKS * 24 : kInSlotBytes;   // uv, w (, w2) per visibility
-    // generator groups: one per stage of the ring at most (see kGroups)
-    constexpr int kGrp0 = kStages < kGroups ? kStages : kGroups;
-    // With two issuers the group count must be even: a group that waits for the release
-    // of stage s - S relies on its previous stage's wait (for stage s - kGrp - S) having
-    // seen stage s - 2S released, which only follows when both stages belong to the same
-    // issuer (each issuer commits in order, the two do not order each other).  An
-    // instance with five groups aliased the parity test and gave up its bounded waits.
-    constexpr int kGrp = (NISS == 2) ? (kGrp0 & ~1) : kGrp0;
-    static_assert(NISS == 1 || kGrp % 2 == 0, "two issuers need an even number of generator groups");
-    static_assert(kGrp <= kStages, "generator groups must not exceed the operand ring depth");
+    using Sh = TcShape<kStages, NISS, MIR, SPLIT>;
+    constexpr int kGrp = Sh::kGroups, kGroupWarps = Sh::kGroupWarps;
+    constexpr int kDrainWarp0 = Sh::kDrainWarp0, kMmaWarp = Sh::kMmaWarp, kInWarp = Sh::kInWarp;
+    constexpr int kMma2Warp = Sh::kMma2Warp;
     static_assert(!SPLIT || MIR <= 2, "split precision covers the plain and mirrored real-weight forms");
     // Two issuers take alternate stages; with an even ring depth every slot (and its release
     // barrier) then belongs to one issuer.  An odd depth makes the two issuing threads commit
@@ -415,7 +340,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
 
-    if (warp < kGrp * kGroupWarps) {
+    if (warp < Sh::kGen) {
         // ------------------------------------------------------------ generators
         const int grp = warp / kGroupWarps, gw = warp % kGroupWarps;
         const int half = it.N / 2;
@@ -425,93 +350,90 @@ __global__ void __launch_bounds__(kThreads, 1)
         // a tile that spans a whole cutout of 64 or 128 pixels only rows N/2 .. N-1 are
         // generated; rows 1 .. N/2 are their conjugates and row 0 the conjugate of the
         // value one step past row N-1.
-        const bool mirror = (MIR == 2) || (MIR == 4) || (MIR == 1 && it.j0 == 0 && it.i0 == 0 && it.ncols == it.N && it.N <= 128 && (it.N & 63) == 0);
+        const bool mirror = whole_cutout<MIR>(it);
         // 32-row chains of the A (128 rows) and B tiles (complex output: A rows past the
         // cutout are skipped)
         const int nA = mirror ? it.N / 64 : (MIR == 5 ? min(4, (it.N - it.j0 + 31) / 32) : 4);
         const int nB = mirror ? it.N / 64 : ncols / 32;
-        uint32_t off8[8];
-        stmatrix_offsets(lane, off8);
         for (int s_i = grp; s_i < nst; s_i += kGrp) {
             const int slot = s_i % kStages;
             const uint32_t ph = (uint32_t)(s_i / kStages) & 1u;
             const int islot = s_i % kInStages;
-            bool ok = wait_bounded(&in_full[islot], (uint32_t)(s_i / kInStages) & 1u, s_abort, err);
-            if (!__all_sync(0xffffffffu, ok)) break;   // warp-uniform exit
+            if (!wait_uniform(&in_full[islot], (uint32_t)(s_i / kInStages) & 1u, s_abort, err)) break;
             const float2 *in_uv = (const float2 *)(smem + L.in_off + islot * kSlot);
             const float2 uvk = in_uv[lane];
             const bool kin = it.k0 + s_i * kKS + lane < it.k1;
             const float2 wk = kin ? in_uv[kKS + lane] : make_float2(0.f, 0.f);
             const float w2k = (MIR == 4 && kin) ? in_uv[2 * kKS + lane].x : 0.f;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&in_empty[islot]);   // the input slot may be refilled
-            if (s_i >= kStages) {
-                ok = wait_bounded(&empty[slot], ph ^ 1u, s_abort, err);
-                if (!__all_sync(0xffffffffu, ok)) break;
-            }
             const uint32_t a_tile = smem_u32(smem + L.a_off + slot * kAStage);
             const uint32_t b_tile = smem_u32(smem + L.b_off + slot * b_stage);
-            if (MIR == 0 && !SPLIT && nA == 4 && nB == 4) {
-                // complex weights on a full 128 x 128 tile: warps 0-1 take two A chains each
-                // (rows 64 gw .. 64 gw + 63), warps 2-3 two B chains each, so the two chains
-                // of a warp share one theta and its step phasors
-                const bool isA = gw < 2;
-                const int c0 = 2 * (gw & 1);
-                const float th = isA ? uvk.y * cell : -uvk.x * cell;
-                const ChainSteps S = chain_steps(th);
-#pragma unroll 1
-                for (int c = c0; c < c0 + 2; ++c) {
-                    if (isA)
-                        gen_chain32_s<BF16, false, false, SPLIT>(S, a_tile + c * 32 * 128, off8, th,
-                                                                 it.j0 + c * 32 - half, wk, true, 0, false, 0,
-                                                                 (uint32_t)kATileBytes);
-                    else
-                        gen_chain32_s<BF16, false, false, SPLIT>(S, b_tile + c * 32 * 128, off8, th,
-                                                                 it.i0 + c * 32 - half, wk, false, 0, false, 0,
-                                                                 bt_stride);
+            const float tv = uvk.y * cell, tu = -uvk.x * cell;
+            auto slot_free = [&]() { return s_i < kStages || wait_uniform(&empty[slot], ph ^ 1u, s_abort, err); };
+            // seeds before the wait for the operand slot, rows after it
+            if (Sh::kTall && MIR == 0 && nA == 4 && nB == 4) {
+                // complex weights on a full 128 x 128 tile: A (weighted column twiddles) in warps 0-1,
+                // 64 rows each; B (conjugated row twiddles) in warps 2-3, conjugate-symmetric where the
+                // tile is a whole cutout (32 generated rows each), else 64 rows each
+                const int role = (gw + grp) & 3;   // each role on every scheduler (warp mod 4)
+                const bool isA = role < 2;
+                if (!isA && it.N == 128) {
+                    const int c = role - 2;
+                    const TwSeeds S = tw_seeds<8>(tu, 32 * c, wk, false);
+                    if (!slot_free()) break;
+                    tw_rows<BF16, 8, true>(S, b_tile + (uint32_t)(64 + 32 * c) * 128u, b_tile + (uint32_t)(64 - 32 * c) * 128u,
+                                           c == 1, b_tile);
+                } else {
+                    const int r0 = 64 * (role & 1);
+                    const TwSeeds S = tw_seeds<16>(isA ? tv : tu, (isA ? it.j0 : it.i0) + r0 - half, wk, isA);
+                    if (!slot_free()) break;
+                    tw_rows<BF16, 16>(S, (isA ? a_tile : b_tile) + (uint32_t)r0 * 128u);
                 }
-            } else
-            for (int ch = gw; ch < nA + nB; ch += kGroupWarps) {
-                if (MIR == 5) {   // A: weighted column twiddles; B: row twiddles, real and imaginary halves
-                    if (ch < nA)
-                        gen_chain32<BF16>(a_tile + ch * 32 * 128, off8, uvk.y * cell, it.j0 + ch * 32 - half, wk, true);
-                    else
-                        gen_chain32<BF16, false, true>(b_tile + (ch - nA) * 32 * 128, off8, -uvk.x * cell,
-                                                       it.i0 + (ch - nA) * 32 - half, wk, false,
-                                                       (uint32_t)ncols * 128u);
-                } else if (MIR == 4) {   // A: unweighted column twiddles; B: weighted row twiddles, both halves
+            } else if (Sh::kTall && MIR == 4 && it.N == 128) {
+                // fused form on a 128-pixel cutout: A in warp 0, B with the Method 1 weights in warp 1,
+                // with the Method 2 weights in warp 2; rows 64 .. 127 and their mirrors
+                const TwSeeds S = tw_seeds<16>(gw ? tu : tv, 0, make_float2(gw == 2 ? w2k : wk.x, 0.f), gw > 0);
+                if (!slot_free()) break;
+                const uint32_t t0 = (gw ? b_tile : a_tile) + (gw == 2 ? 128u * 128u : 0u);
+                tw_rows<BF16, 16, true>(S, t0 + 64 * 128, t0 + 64 * 128, true, t0);
+            } else {
+                bool free = false;
+                // units: the 32-row chains of A, then those of B (in the fused form once per weight)
+                constexpr int kBW = MIR == 4 ? 2 : 1;
+                for (int ch = gw; ch < nA + kBW * nB; ch += kGroupWarps) {
                     const bool isA = ch < nA;
-                    const int c = isA ? ch : ch - nA;
-                    const int R0 = half + 32 * c;
-                    if (isA)
-                        gen_chain32<BF16, true>(a_tile + (uint32_t)R0 * 128u, off8, uvk.y * cell, 32 * c, wk, false,
-                                                a_tile + (uint32_t)(it.N - R0) * 128u, c == nA - 1, a_tile);
-                    else
-                        gen_chain32_dual<BF16>(b_tile + (uint32_t)R0 * 128u, b_tile + (uint32_t)(it.N - R0) * 128u,
-                                               (uint32_t)it.N * 128u, -uvk.x * cell, 32 * c, wk.x, w2k, c == nB - 1,
-                                               b_tile);
-                } else if (mirror) {   // rows R0 .. R0+31 (R0 = N/2 + 32 c) and their mirrors N - R0 - r
-                    const bool isA = ch < nA;
-                    const int c = isA ? ch : ch - nA;
-                    const int R0 = half + 32 * c;
+                    const int c = isA ? ch : (ch - nA) / kBW;
                     const uint32_t tile = isA ? a_tile : b_tile;
-                    gen_chain32<BF16, true, false, SPLIT>(tile + (uint32_t)R0 * 128u, off8,
-                                                          isA ? uvk.y * cell : -uvk.x * cell, 32 * c, wk, isA,
-                                                          tile + (uint32_t)(it.N - R0) * 128u, c == nA - 1, tile,
-                                                          isA ? (uint32_t)kATileBytes : bt_stride);
-                } else if (ch < nA) {   // weighted column twiddles c_k[j], rows j = j0 + 32 ch + r
-                    gen_chain32<BF16, false, false, SPLIT>(a_tile + ch * 32 * 128, off8, uvk.y * cell,
-                                                           it.j0 + ch * 32 - half, wk, true, 0, false, 0,
-                                                           (uint32_t)kATileBytes);
-                } else {                // conjugated row twiddles (a_r, -a_i), rows i = i0 + 32 (ch - nA) + r
-                    gen_chain32<BF16, false, false, SPLIT>(b_tile + (ch - nA) * 32 * 128, off8, -uvk.x * cell,
-                                                           it.i0 + (ch - nA) * 32 - half, wk, false, 0, false, 0,
-                                                           bt_stride);
+                    if (MIR == 4 || mirror) {
+                        // rows R0 .. R0 + 31 (R0 = N/2 + 32 c) and their mirrors N - R0 - r; the fused form
+                        // weights the row twiddles (both halves of B), the others the column twiddles
+                        const int R0 = half + 32 * c;
+                        const bool second = MIR == 4 && !isA && ((ch - nA) & 1);
+                        const float2 wv = MIR == 4 ? make_float2(second ? w2k : wk.x, 0.f) : wk;
+                        const TwSeeds S = tw_seeds<8>(isA ? tv : tu, 32 * c, wv, isA != (MIR == 4));
+                        if (!free && !(free = slot_free())) break;
+                        const uint32_t t0 = tile + (second ? (uint32_t)it.N * 128u : 0u);
+                        tw_rows<BF16, 8, true, false, SPLIT>(S, t0 + (uint32_t)R0 * 128u,
+                                                             t0 + (uint32_t)(it.N - R0) * 128u, c == it.N / 64 - 1, t0, 0,
+                                                             isA ? (uint32_t)kATileBytes : bt_stride);
+                    } else {   // weighted column twiddles c_k[j] (A) or conjugated row twiddles (a_r, -a_i) (B)
+                        const TwSeeds S = tw_seeds<8>(isA ? tv : tu, (isA ? it.j0 : it.i0) + 32 * c - half, wk, isA);
+                        if (!free && !(free = slot_free())) break;
+                        if (MIR == 5 && !isA)
+                            tw_rows<BF16, 8, false, true>(S, tile + c * 32 * 128, 0, false, 0, (uint32_t)ncols * 128u);
+                        else
+                            tw_rows<BF16, 8, false, false, SPLIT>(S, tile + c * 32 * 128, 0, false, 0, 0,
+                                                                  isA ? (uint32_t)kATileBytes : bt_stride);
+                    }
                 }
+                if (!free && !slot_free()) break;
             }
             fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&full[slot]);
+            if (lane == 0) {
+                mbar_arrive(&full[slot]);
+                // the input slot is released only after the stores that depend on its values
+                mbar_arrive(&in_empty[islot]);
+            }
         }
     } else if (warp == kMmaWarp || (NISS == 2 && warp == kMma2Warp)) {
         // ------------------------------------------------------------ MMA issue
@@ -520,45 +442,49 @@ __global__ void __launch_bounds__(kThreads, 1)
         // [d kRange, (d + 1) kRange) and uses buffer b = d mod 2.
         {
             const int q = (warp == kMmaWarp) ? 0 : 1;
-            // The issue path is short and warp-uniform (umma_f16_x4): slot, phase and range
-            // by increment, descriptors by adding the slot offset to the address field.
+            // The issue path is short and warp-uniform (umma_f16_x4); among the generators its
+            // instructions count more than the tensor core's time.
             const uint32_t el = elect_one();
             const uint32_t idesc = warp_uniform(idesc_f16(128, kBMul * ncols, BF16));
             const uint32_t ad0 = warp_uniform(desc_lo(smem_u32(smem + L.a_off)));
             const uint32_t bd0 = warp_uniform(desc_lo(smem_u32(smem + L.b_off)));
             const uint32_t b_units = warp_uniform(b_stage >> 4), tm0 = warp_uniform(tmem);
             const uint32_t cols = warp_uniform(acc_cols);
-            int slot = q, r = q, d = 0;
+            // one ring round per outer iteration, unrolled over this issuer's slots
+            const uint32_t adq = ad0 + (uint32_t)q * (kAStage >> 4), bdq = bd0 + (uint32_t)q * b_units;
+            int r = q, d = 0;
             uint32_t ph = 0;
-            for (int s_i = q; s_i < nst; s_i += NISS) {
-                if (!__all_sync(0xffffffffu, wait_bounded(&full[slot], ph, s_abort, err))) break;
-                const int b = d & 1;
-                if (r == q && d >= 2 &&   // first own stage of a range: the buffer's last drain is done
-                    !__all_sync(0xffffffffu,
-                                wait_bounded(&acc_empty[b], (uint32_t)((d >> 1) - 1) & 1u, s_abort, err)))
-                    break;
-                tc_fence_after();
-                const uint32_t ad = ad0 + (uint32_t)slot * (kAStage >> 4);
-                const uint32_t bd = bd0 + (uint32_t)slot * b_units;
-                const uint32_t dt = tm0 + (uint32_t)(2 * q + b) * cols;
-                // a range's first MMA clears the buffer, except issuer 0's from range 2 on:
-                // the drain has left the compensation of the running sum there
-                umma_f16_x4(dt, ad, bd, idesc, (r != q || (SPLIT && q == 0 && d >= 2)) ? 1u : 0u, el);
-                if (SPLIT) {   // A_hi B_lo, then A_lo B_hi
-                    umma_f16_x4(dt, ad, bd + (bt_stride >> 4), idesc, 1u, el);
-                    umma_f16_x4(dt, ad + (kATileBytes >> 4), bd, idesc, 1u, el);
-                }
-                umma_commit_elected(&empty[slot], el);
-                r += NISS;
-                if (r >= kRange || s_i + NISS >= nst) umma_commit_elected(&acc_full[2 * q + b], el);
-                if (r >= kRange) {
-                    r -= kRange;
-                    ++d;
-                }
-                slot += NISS;
-                if (slot >= kStages) {
-                    slot -= kStages;
-                    ph ^= 1u;
+            bool stop = false;
+            for (int s0 = q; s0 < nst && !stop; s0 += kStages, ph ^= 1u) {
+#pragma unroll
+                for (int i = 0; i < kStages / NISS; ++i) {
+                    const int s_i = s0 + NISS * i;
+                    if (s_i >= nst || stop) break;
+                    const int b = d & 1;
+                    if (r == q && d >= 2 &&   // first own stage of a range: the buffer's last drain is done
+                        !wait_uniform(&acc_empty[b], (uint32_t)((d >> 1) - 1) & 1u, s_abort, err)) {
+                        stop = true;
+                        break;
+                    }
+                    if (!wait_uniform(&full[q + NISS * i], ph, s_abort, err)) { stop = true; break; }
+                    tc_fence_after();
+                    const uint32_t ad = adq + (uint32_t)(NISS * i) * (kAStage >> 4);
+                    const uint32_t bd = bdq + (uint32_t)(NISS * i) * b_units;
+                    const uint32_t dt = tm0 + (uint32_t)(2 * q + b) * cols;
+                    // a range's first MMA clears the buffer, except issuer 0's from range 2 on:
+                    // the drain has left the compensation of the running sum there
+                    umma_f16_x4(dt, ad, bd, idesc, (r != q || (SPLIT && q == 0 && d >= 2)) ? 1u : 0u, el);
+                    if (SPLIT) {   // A_hi B_lo, then A_lo B_hi
+                        umma_f16_x4(dt, ad, bd + (bt_stride >> 4), idesc, 1u, el);
+                        umma_f16_x4(dt, ad + (kATileBytes >> 4), bd, idesc, 1u, el);
+                    }
+                    umma_commit_elected(&empty[q + NISS * i], el);
+                    r += NISS;
+                    if (r >= kRange || s_i + NISS >= nst) umma_commit_elected(&acc_full[2 * q + b], el);
+                    if (r >= kRange) {
+                        r -= kRange;
+                        ++d;
+                    }
                 }
             }
             // all issued MMAs complete before TMEM is released (waited for even after
@@ -592,11 +518,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 wait_bounded(&in_full[s_i % kInStages], (uint32_t)(s_i / kInStages) & 1u, &no_abort, err);
         }
         __syncwarp();
+    } else if (warp < kDrainWarp0) {
+        // fills the generator warps up to a multiple of four: idle
     } else if (warp == kMma2Warp) {
         // second issuer, idle with one issuer (NISS == 1): it must not join the drain
         // warps (lane quarters 0-3, four arrivals per accumulator release)
-    } else if (warp < kGenWarps) {
-        // generator warps beyond the ring depth's groups (split precision): idle
     } else {
         // ------------------------------------------------------------ drain
         // The partial cutout is stored transposed (element (j, i) at i N + j), so the 32
@@ -609,6 +535,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool row_ok = j < it.N;
         const int ncol_valid = min(ncols, it.N - it.i0);
         float *dst2 = dst + part2;   // second cutout of the fused form
+        // signs of the operand rows (row_sign; mirrored tiles count from the cutout's centre)
+        const bool mirror = whole_cutout<MIR>(it);
+        const bool mirror_b = mirror || (Sh::kTall && MIR == 0 && it.N == 128);
+        auto sign_of = [&](int r, bool m) { return row_sign(m ? abs(r - it.N / 2) : r); };
+        const float rs = sign_of(q * 32 + lane, mirror);
         if (nst == 0) {
             if (row_ok)
                 for (int c = 0; c < ncol_valid; ++c) {
@@ -641,6 +572,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                     for (int e = 0; e < 16; ++e) v[e] += v2[e];
                 }
+                float sg[4];   // row sign times the sign of columns c0 + e (e mod 4)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sg[e] = rs * sign_of(cb + e, mirror_b);
+#pragma unroll
+                for (int e = 0; e < 16; ++e) v[e] *= sg[e & 3];
                 if (SPLIT) {
                     float sv[16], cv[16];   // running sum; compensation for the buffer's next range
 #pragma unroll
@@ -656,21 +592,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                             if (cb + e < ncol_valid) dd[(cb + e) * cstride] = v[e];
                     }
                     // issuer 0's buffer b is accumulated on again by range d + 2
-                    if (d + 2 < ndrain) tmem_st16(ta + (uint32_t)c0, cv);
+                    if (d + 2 < ndrain) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) cv[e] *= sg[e & 3];
+                        tmem_st16(ta + (uint32_t)c0, cv);
+                    }
                     continue;
                 }
+                // The first range stores, later ones add by reductions, which return nothing
+                // (one thread owns each element, so the sum has a fixed order): a load, an add and
+                // a store per element took an L2 round trip per eight.
                 if (row_ok) {
-                    // eight loads in flight before their stores (one L2 round trip per eight)
 #pragma unroll
-                    for (int h = 0; h < 16; h += 8) {
-                        float o[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            o[e] = (d > 0 && cb + h + e < ncol_valid) ? dd[(cb + h + e) * cstride] : 0.f;
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (cb + h + e < ncol_valid) dd[(cb + h + e) * cstride] = o[e] + v[h + e];
-                    }
+                    for (int e = 0; e < 16; ++e)
+                        if (cb + e < ncol_valid) {
+                            if (d == 0) dd[(cb + e) * cstride] = v[e];
+                            else red_add(dd + (cb + e) * cstride, v[e]);
+                        }
                 }
             }
             tc_fence_before();
@@ -794,7 +732,7 @@ static cudaError_t launch_tc_t(const DevObs &o, const float2 *w, int64_t ldw, co
     cudaError_t e = cudaFuncSetAttribute(k_psf_tc<BF16, S, NISS, MIR, SPLIT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    k_psf_tc<BF16, S, NISS, MIR, SPLIT><<<nitems, kThreads, bytes, st>>>(o.uv, w, ldw, items, ncols_max, cell,
+    k_psf_tc<BF16, S, NISS, MIR, SPLIT><<<nitems, TcShape<S, NISS, MIR, SPLIT>::kThreads, bytes, st>>>(o.uv, w, ldw, items, ncols_max, cell,
                                                                           partial, split_stride, err, w2, part2);
     return cudaGetLastError();
 }

@@ -268,6 +268,35 @@ static __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
 }
 
 
+// Nearest integer by adding 1.5 * 2^23 (|x| < 2^22; the conversion unit's rounding
+// instruction runs at a quarter of the FP32 rate).
+static __device__ __forceinline__ float nearest(float x) { return __fadd_rn(__fadd_rn(x, 12582912.0f), -12582912.0f); }
+
+// exp(2 pi i x) as cis_turns, without the conversion unit.
+static __device__ __forceinline__ float2 cis_fast(float x) {
+    float2 z;
+    __sincosf(6.28318530717958647f * (x - nearest(x)), &z.y, &z.x);
+    return z;
+}
+
+// cos and sin of the step 2 pi x from the half angle: the recurrence x_{n+1} = 2 cos(step) x_n
+// - x_{n-1} amplifies an error of cos(step) by up to the square of its length where the step
+// is small, and 1 - 2 sin^2 (2 cos^2 - 1 beyond a quarter turn) keeps that error at the
+// rounding of 1.
+static __device__ __forceinline__ void step_phasor(float x, float &re, float &im) {
+    const float f = x - nearest(x);
+    float s, c;
+    __sincosf(3.14159265358979324f * f, &s, &c);
+    re = fabsf(f) < 0.25f ? fmaf(-2.0f * s, s, 1.0f) : fmaf(2.0f * c, c, -1.0f);
+    im = 2.0f * s * c;
+}
+
+static __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// Sign with which the recurrences carry row r of an operand tile (pieces of 8 or 16 rows
+// seeded at their middle): + - - + repeated; the output applies it.
+static __host__ __device__ __forceinline__ constexpr float row_sign(int r) { return ((r + 1) & 2) ? -1.0f : 1.0f; }
+
 // Four 8x8 b16 matrices from registers to shared memory.  Lane t holds, per matrix,
 // the 32-bit pair at matrix row t/4, columns 2(t%4), 2(t%4)+1; lanes 8m..8m+7 give
 // the 16-byte row addresses of matrix m.  With one K-major 128-byte operand row per
@@ -277,6 +306,14 @@ static __device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t v0, 
                                                    uint32_t v3) {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(v0), "r"(v1),
                  "r"(v2), "r"(v3)
+                 : "memory");
+}
+
+template <int OFF>
+static __device__ __forceinline__ void stmatrix_x4_at(uint32_t saddr, uint32_t v0, uint32_t v1, uint32_t v2,
+                                                      uint32_t v3) {   // at saddr + OFF bytes
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0 + %5], {%1, %2, %3, %4};" ::"r"(saddr), "r"(v0),
+                 "r"(v1), "r"(v2), "r"(v3), "n"(OFF)
                  : "memory");
 }
 
