@@ -366,35 +366,61 @@ cudaError_t launch_zero_cutouts(float *out, const int64_t *offs, const int32_t *
 }
 
 // --------------------------------------------------------------- FP32 contraction
-// One CTA per (64 x 64 tile, visibility range); the tile body is fp32t::tile_sum.
-__global__ void __launch_bounds__(256) k_psf_fp32(const float2 *__restrict__ uv, const float2 *__restrict__ uv_lo,
-                                                  const float2 *__restrict__ w, int64_t ldw, int32_t nvis,
-                                                  const Tile *__restrict__ tiles, int32_t kper, float2 cell,
-                                                  float *__restrict__ partial, int64_t split_stride) {
-    __shared__ __align__(16) float2 sa[fp32t::kKC][fp32t::kT];   // row (l) twiddles
-    __shared__ __align__(16) float2 sc[fp32t::kKC][fp32t::kT];   // weighted column (m) twiddles
+// One CTA per (tile, visibility range); the tile body is fp32t::tile_block.
+template <int A, int B>
+__global__ void __launch_bounds__(256, 1)
+    k_psf_fp32(const float2 *__restrict__ uv, const float2 *__restrict__ uv_lo, const float2 *__restrict__ w, int64_t ldw,
+               int32_t nvis, const Tile *__restrict__ tiles, int32_t kper, float2 cell, float *__restrict__ partial,
+               int64_t split_stride) {
+    extern __shared__ __align__(16) float fp32_smem[];
     const Tile t = tiles[blockIdx.x];
-    const int split = blockIdx.y;
-    const int32_t kbeg = split * kper;
-    const int32_t kend = min(nvis, kbeg + kper);
-    const float2 *wp = w + (int64_t)t.slot * ldw;
-    float tot[4][4];
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-        for (int a = 0; a < 4; ++a) tot[b][a] = 0.f;
-    fp32t::tile_sum(uv, uv_lo, kbeg, kend, t.N, t.i0, t.j0, cell, [&](int32_t k) { return wp[k]; }, sa, sc, tot);
-    fp32t::tile_store(partial + (int64_t)split * split_stride + t.out_off, t.N, t.i0, t.j0, tot);
+    const int32_t kbeg = blockIdx.y * kper;
+    fp32t::tile_block<A, B>(fp32_smem, uv, uv_lo, w + (int64_t)t.slot * ldw, kbeg, min(nvis, kbeg + kper), t.N, t.i0, t.j0,
+                            cell, partial + (int64_t)blockIdx.y * split_stride + t.out_off);
+}
+
+// Tile shapes (8 A x 8 B pixels) and their relative cost per pixel-visibility term (larger
+// blocks per thread load fewer operands per FMA): a call takes the shape with the least
+// padded work over its cutouts.
+static const struct { int A, B; double cost; } kFp32Shapes[] = {{8, 8, 1.0}, {10, 5, 1.1}, {6, 6, 1.15}, {4, 4, 1.5}};
+
+int fp32_shape(const int32_t *npix, int npos, int *ti, int *tj) {
+    int best = 0;
+    double best_cost = 0.0;
+    for (int s = 0; s < 4; ++s) {
+        const int Ti = 8 * kFp32Shapes[s].A, Tj = 8 * kFp32Shapes[s].B;
+        double c = 0.0;
+        for (int p = 0; p < npos; ++p)
+            c += (double)((npix[p] + Ti - 1) / Ti * Ti) * ((npix[p] + Tj - 1) / Tj * Tj) * kFp32Shapes[s].cost;
+        if (s == 0 || c < best_cost) { best = s; best_cost = c; }
+    }
+    *ti = 8 * kFp32Shapes[best].A;
+    *tj = 8 * kFp32Shapes[best].B;
+    return best;
+}
+
+template <int A, int B>
+static cudaError_t launch_fp32_t(const DevObs &o, const float2 *w, int64_t ldw, const Tile *tiles, int ntiles, int nsplit,
+                                 int32_t kper, double cell, float *partial, int64_t split_stride, cudaStream_t st) {
+    constexpr size_t smem = fp32t::Block<A, B>::kSmem;
+    cudaError_t e = cudaFuncSetAttribute(k_psf_fp32<A, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_psf_fp32<A, B><<<dim3(ntiles, nsplit), 256, smem, st>>>(o.uv, o.uv_lo, w, ldw, o.nvis, tiles, kper,
+                                                              fp32t::cell_pair(cell), partial, split_stride);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_psf_fp32(const DevObs &o, const float2 *w, int64_t ldw, const Tile *tiles, int ntiles,
-                            int nsplit, int32_t kper, double cell, float *partial, int64_t split_stride,
+                            int nsplit, int32_t kper, double cell, float *partial, int64_t split_stride, int shape,
                             cudaStream_t st) {
     if (ntiles <= 0) return cudaSuccess;
-    dim3 grid(ntiles, nsplit);
-    k_psf_fp32<<<grid, 256, 0, st>>>(o.uv, o.uv_lo, w, ldw, o.nvis, tiles, kper, fp32t::cell_pair(cell), partial,
-                                     split_stride);
-    return cudaGetLastError();
+    switch (shape) {
+        case 0: return launch_fp32_t<8, 8>(o, w, ldw, tiles, ntiles, nsplit, kper, cell, partial, split_stride, st);
+        case 1: return launch_fp32_t<10, 5>(o, w, ldw, tiles, ntiles, nsplit, kper, cell, partial, split_stride, st);
+        case 2: return launch_fp32_t<6, 6>(o, w, ldw, tiles, ntiles, nsplit, kper, cell, partial, split_stride, st);
+        case 3: return launch_fp32_t<4, 4>(o, w, ldw, tiles, ntiles, nsplit, kper, cell, partial, split_stride, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // --------------------------------------------------------------- FP32 FMA rate
@@ -480,25 +506,47 @@ int selftest_fma_rate(int packed, double *flops_per_s) {
 }
 
 // --------------------------------------------------------------- split reduction
-// One block row per position; the partial sums of each pixel are added in float64
-// in split order (deterministic).  Partials use chunk-local packed offsets, the
+// One block row per position; 32 pixels per block, the splits of a pixel shared by eight
+// threads (splits s mod 8, four loads in flight each) and their float64 sums added in a
+// fixed order (deterministic).  One thread per pixel walked up to 152 splits one L2 round
+// trip after another (24 us per cutout).  Partials use chunk-local packed offsets, the
 // output the caller's offsets.
 __global__ void __launch_bounds__(256) k_reduce(const float *__restrict__ partial, int nsplit,
                                                 int64_t stride, const int64_t *__restrict__ loc_offs,
                                                 const int64_t *__restrict__ out_offs,
                                                 const int32_t *__restrict__ npix, int transposed,
                                                 float *__restrict__ out) {
+    __shared__ double sum[8][32];
     const int p = blockIdx.y;
     const int N = npix[p];
     const int64_t n2 = (int64_t)N * N;
     const float *src = partial + loc_offs[p];
     float *dst = out + out_offs[p];
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += (int64_t)gridDim.x * blockDim.x) {
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int64_t q0 = (int64_t)blockIdx.x * 32; q0 < n2; q0 += (int64_t)gridDim.x * 32) {
+        const int64_t q = q0 + tx;
         double s = 0.0;
-        for (int sp = 0; sp < nsplit; ++sp) s += (double)src[(int64_t)sp * stride + q];
-        // transposed partials hold (j, i) at q = i N + j
-        const int64_t o = transposed ? (q % N) * N + q / N : q;
-        dst[o] = (float)s;
+        if (q < n2) {
+            int sp = ty;
+            for (; sp + 24 < nsplit; sp += 32) {
+                float v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = src[(int64_t)(sp + 8 * u) * stride + q];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s += (double)v[u];
+            }
+            for (; sp < nsplit; sp += 8) s += (double)src[(int64_t)sp * stride + q];
+        }
+        sum[ty][tx] = s;
+        __syncthreads();
+        if (ty == 0 && q < n2) {
+#pragma unroll
+            for (int u = 1; u < 8; ++u) s += sum[u][tx];
+            // transposed partials hold (j, i) at q = i N + j
+            const int64_t o = transposed ? (q % N) * N + q / N : q;
+            dst[o] = (float)s;
+        }
+        __syncthreads();
     }
 }
 
@@ -506,7 +554,7 @@ cudaError_t launch_reduce(const float *partial, int nsplit, int64_t stride, cons
                           const int64_t *out_offs, const int32_t *npix, int npos, int transposed, float *out,
                           cudaStream_t st) {
     if (npos <= 0) return cudaSuccess;
-    dim3 grid(64, npos);
+    dim3 grid((unsigned)std::max(16, 512 / npos), npos);
     k_reduce<<<grid, 256, 0, st>>>(partial, nsplit, stride, loc_offs, out_offs, npix, transposed, out);
     return cudaGetLastError();
 }

@@ -33,8 +33,8 @@ static __device__ __align__(256) float g_noalloc_partial[kNaScratchFloats];
 
 __global__ void __launch_bounds__(256) k_noalloc_exact(DevObs o, uint32_t flags, float4 L, int N, float2 cell,
                                                        int32_t kper, float *__restrict__ partial) {
-    __shared__ __align__(16) float2 sa[fp32t::kKC][fp32t::kT];
-    __shared__ __align__(16) float2 sc[fp32t::kKC][fp32t::kT];
+    __shared__ __align__(16) float2 sa[fp32t::kKC][fp32t::kTP];
+    __shared__ __align__(16) float2 sc[fp32t::kKC][fp32t::kTP];
     const int ntx = (N + fp32t::kT - 1) / fp32t::kT;
     const int i0 = (blockIdx.x % ntx) * fp32t::kT, j0 = (blockIdx.x / ntx) * fp32t::kT;
     const int split = blockIdx.y;

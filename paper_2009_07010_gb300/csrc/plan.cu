@@ -540,6 +540,23 @@ constexpr size_t kWeightBudget = size_t(4) << 30;   // weights of one position c
 constexpr size_t kW16Budget = size_t(4) << 30;      // FP16 weights of one batched chunk (bytes)
 constexpr int kKrMinGroup = 32;                     // positions of one size for the batched form
 
+// Visibility ranges of `base` tiles so that base x ranges CTAs (one per SM) fill whole waves:
+// the count that minimises waves x (range + per-CTA overhead), in visibilities.  Small
+// observations are spread over the whole chip (ranges of 8192 and 4096 visibilities at
+// least left a 172 800-visibility cutout on 22 and 43 of the 152 SMs), and a count just
+// above a whole wave is avoided.
+int best_splits(int64_t base, int64_t K, int nsm, int64_t overhead, int64_t least) {
+    const int64_t most = std::max<int64_t>(1, std::min<int64_t>((K + least - 1) / least, 4 * (int64_t)nsm));
+    int64_t best = 1, best_cost = INT64_MAX;
+    for (int64_t n = 1; n <= most; ++n) {
+        const int64_t cost = ((base * n + nsm - 1) / nsm) * ((K + n - 1) / n + overhead);
+        if (cost < best_cost) { best_cost = cost; best = n; }
+    }
+    return (int)best;
+}
+constexpr int64_t kTcOverhead = 640, kTcLeast = 512;       // k_psf_tc: pipeline fill, drain and set-up
+constexpr int64_t kFp32Overhead = 192, kFp32Least = 256;   // k_psf_fp32
+
 // One size group of the batched form: positions idx (batch indices) of cutout size N.
 struct KrGroup {
     int N;
@@ -845,17 +862,17 @@ int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cud
 
         std::vector<Tile> tiles;
         std::vector<TcItem> items;
-        int nsplit = 1, ncols_max = 16;
+        int nsplit = 1, ncols_max = 16, shape = 0;
         int32_t kper = (int32_t)K;
         if (!tc) {
+            int ti = 64, tj = 64;
+            shape = fp32_shape(&h.npix[c0], cn, &ti, &tj);
             for (int i = 0; i < cn; ++i) {
                 const int N = h.npix[c0 + i];
-                for (int j0 = 0; j0 < N; j0 += 64)
-                    for (int i0 = 0; i0 < N; i0 += 64) tiles.push_back(Tile{i, N, i0, j0, loc[i]});
+                for (int j0 = 0; j0 < N; j0 += tj)
+                    for (int i0 = 0; i0 < N; i0 += ti) tiles.push_back(Tile{i, N, i0, j0, loc[i]});
             }
-            const int64_t target = 4LL * p->nsm;
-            nsplit = (int)std::max<int64_t>(1, std::min<int64_t>((target + tiles.size() - 1) / tiles.size(),
-                                                                  (K + 4095) / 4096));
+            nsplit = best_splits((int64_t)tiles.size(), K, p->nsm, kFp32Overhead, kFp32Least);
             kper = (int32_t)(((K + nsplit - 1) / nsplit + 31) / 32 * 32);
             nsplit = (int)((K + kper - 1) / kper);
         } else {
@@ -871,9 +888,7 @@ int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cud
                         base.push_back(TcItem{i, N, j0, i0, nc, 0, 0, 0, loc[i]});
                     }
             }
-            const int64_t target = p->nsm;
-            nsplit = (int)std::max<int64_t>(1, std::min<int64_t>((target + base.size() - 1) / base.size(),
-                                                                  (K + 8191) / 8192));
+            nsplit = best_splits((int64_t)base.size(), K, p->nsm, kTcOverhead, kTcLeast);
             kper = (int32_t)(((K + nsplit - 1) / nsplit + 31) / 32 * 32);
             nsplit = (int)((K + kper - 1) / kper);
             for (int sp = 0; sp < nsplit; ++sp)
@@ -944,7 +959,7 @@ int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cud
         }
         if (!tc) {
             PSF_TRY(launch_psf_fp32(p->d, w, ldw, (const Tile *)(dm + m.off_tiles), (int)tiles.size(), nsplit,
-                                    kper, h.cell, part, stride, st));
+                                    kper, h.cell, part, stride, shape, st));
         } else {
             // the approximations' weights are real unless windowed (Eqs. 15-16: a window's
             // transform is complex in general)
@@ -1018,7 +1033,7 @@ int run_forward_uvimg(psf_plan_s *p, const psf_batch_t *b, float *out_uv, float 
             const int N = h.npix[c0 + i];
             base.push_back(TcItem{i, N, 0, 0, N, 0, 0, 0, loc[i]});
         }
-        int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>((p->nsm + cn - 1) / cn, (K + 8191) / 8192));
+        int nsplit = best_splits(cn, K, p->nsm, kTcOverhead, kTcLeast);
         const int32_t kper = (int32_t)(((K + nsplit - 1) / nsplit + 31) / 32 * 32);
         nsplit = (int)((K + kper - 1) / kper);
         for (int sp = 0; sp < nsplit; ++sp)
@@ -1107,7 +1122,7 @@ int run_forward_cplx(psf_plan_s *p, int method, const BatchHost &h, float *out, 
             ncols_max = std::max(ncols_max, nc);
             base.push_back(TcItem{i, N, 0, 0, nc, 0, 0, 0, loc[i]});
         }
-        int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>((p->nsm + cn - 1) / cn, (K + 8191) / 8192));
+        int nsplit = best_splits(cn, K, p->nsm, kTcOverhead, kTcLeast);
         const int32_t kper = (int32_t)(((K + nsplit - 1) / nsplit + 31) / 32 * 32);
         nsplit = (int)((K + kper - 1) / kper);
         for (int sp = 0; sp < nsplit; ++sp)

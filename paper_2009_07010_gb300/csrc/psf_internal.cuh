@@ -63,7 +63,10 @@ cudaError_t launch_weights(const DevObs &o, int method, uint32_t flags, const fl
 // FP32 CUDA-core contraction; partial[split * split_stride + out_off + j*N + i].
 cudaError_t launch_psf_fp32(const DevObs &o, const float2 *w, int64_t ldw, const Tile *tiles,
                             int ntiles, int nsplit, int32_t kper, double cell, float *partial,
-                            int64_t split_stride, cudaStream_t st);
+                            int64_t split_stride, int shape, cudaStream_t st);
+// Tile shape of the FP32 contraction for a set of cutouts (an index for launch_psf_fp32) and
+// its size in columns and rows.
+int fp32_shape(const int32_t *npix, int npos, int *ti, int *tj);
 // out[out_off_p + q] = sum_s partial[s * stride + loc_off_p + q'] (float64 sum), where
 // q' = q for row-major partials and q' = i N + j for q = j N + i when `transposed`.
 cudaError_t launch_reduce(const float *partial, int nsplit, int64_t stride, const int64_t *loc_offs,
