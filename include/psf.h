@@ -283,11 +283,9 @@ typedef struct {
  * to it (it is not cleared).  comp_pix_dev / comp_flux_dev: device int32 / float32
  * [max_iter] or NULL: per iteration the peak pixel index y * nl + x and the subtracted
  * flux gain * I_D(l0).  *niter_out (host, may be NULL): iterations performed.  With
- * PSF_METHOD_IMG_GRID every step stays on the device and the host reads the loop
- * record once per 64 queued iterations (after the first 64, replayed as one CUDA graph
- * on a private stream); the other methods read the peak record back
- * each iteration to place the cutout (with PSF_CLEAN_FACET_PSF every method stays on
- * the device after the one PSF evaluation).  Errors: PSF_EINVAL (sizes, gain, method, NULL
+ * PSF_METHOD_IMG_GRID, and with PSF_CLEAN_FACET_PSF after the one PSF evaluation, the
+ * loop runs inside a kernel and the host reads its record once per 1024 iterations; the
+ * other methods read the peak record back each iteration to place the cutout.  Errors: PSF_EINVAL (sizes, gain, method, NULL
  * residual), PSF_EUNSUPPORTED (a cutout size the method does not support,
  * PSF_COMPLEX_OUT), and those of the PSF calls. */
 int psf_clean(psf_plan_t plan, const psf_clean_t *cfg, float *residual_dev, float *model_dev,

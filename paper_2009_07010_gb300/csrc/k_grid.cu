@@ -489,6 +489,305 @@ cudaError_t launch_img_grid_n(const float4 *G, const GridPos *pos, int npos, flo
     return cudaGetLastError();
 }
 
+// ------------------------------------------------------------------ CLEAN loop
+// Algorithm 2's loop on one cluster of eight CTAs, many iterations per launch.  As separate
+// kernels an iteration took 27.6 us on a 2048^2 image with N = 128: the argmax read the whole
+// image (5.7 us), one CTA evaluated the PSF (15 us), and four launches followed one another.
+// Here
+//   * the peak is found from per-row maxima: the window of an iteration changes N rows, and
+//     each CTA renews the maxima of its own N/8 of them (per 64-pixel segment, then per row);
+//   * the PSF's columns, then its rows, are shared by the CTAs, exchanged through distributed
+//     shared memory, with k_img_grid's operations per element (bit-identical values);
+//   * cluster barriers (three per iteration) order everything.
+// 10.9 us per iteration.  FACET: one given PSF (P, any even N) instead of the gridded one.
+// Maxima are 64-bit keys as k_clean_argmax forms them (value, then the first pixel).
+constexpr int kClCtas = 8, kClThreads = 256, kClSeg = 64;
+
+__device__ __forceinline__ unsigned long long clean_key(float v, int64_t pix) {
+    const unsigned int u = __float_as_uint(v);
+    const unsigned int o = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    return ((unsigned long long)o << 32) | (unsigned long long)(0xffffffffu - (unsigned int)pix);
+}
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long k) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, k, o);
+        k = x > k ? x : k;
+    }
+    return k;
+}
+// Keys of the segments s0 .. s1 of row y, then of the row, by one warp.  Residual and keys
+// are read past L1: other CTAs of the cluster write them.
+__device__ __forceinline__ void clean_row_keys(const float *res, int y, int nl, int nseg, int s0, int s1,
+                                               unsigned long long *seg, unsigned long long *row) {
+    const int lane = threadIdx.x & 31;
+    for (int s = s0; s <= s1; ++s) {
+        unsigned long long k = 0;
+#pragma unroll
+        for (int h = 0; h < kClSeg; h += 32) {
+            const int x = s * kClSeg + h + lane;
+            if (x < nl) {
+                const int64_t pix = (int64_t)y * nl + x;
+                const unsigned long long q = clean_key(__ldcg(res + pix), pix);
+                k = q > k ? q : k;
+            }
+        }
+        k = warp_max(k);
+        if (lane == 0) seg[(int64_t)y * nseg + s] = k;
+    }
+    __syncwarp();
+    unsigned long long k = 0;
+    for (int s = lane; s < nseg; s += 32) {
+        const unsigned long long q = __ldcg(seg + (int64_t)y * nseg + s);
+        k = q > k ? q : k;
+    }
+    k = warp_max(k);
+    if (lane == 0) row[y] = k;
+}
+
+__global__ void __launch_bounds__(256) k_clean_keys(const float *__restrict__ res, int nl, int nm, int nseg,
+                                                    unsigned long long *__restrict__ seg,
+                                                    unsigned long long *__restrict__ row) {
+    for (int y = blockIdx.x * 8 + (threadIdx.x >> 5); y < nm; y += gridDim.x * 8)
+        clean_row_keys(res, y, nl, nseg, 0, nseg - 1, seg, row);
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, int rank) {   // p's address in CTA `rank`
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, float2 v) {
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ float cluster_load(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+template <int N, bool FACET>
+__global__ void __launch_bounds__(kClThreads) __cluster_dims__(kClCtas, 1, 1)
+    k_clean_loop(const float4 *__restrict__ G, const float *__restrict__ Pf, int nf, float *res, float *__restrict__ model,
+                 CleanState *st, int nl, int nm, double cell, double lc, double mc, float gain, float threshold, int max_iter,
+                 int chunk, int literal, int32_t *__restrict__ comp_pix, float *__restrict__ comp_flux,
+                 unsigned long long *seg, unsigned long long *row) {
+    using F = GridFft<N>;
+    constexpr int M = N / 2, LD = M + 1, R1 = F::R1, R2 = F::R2, Q1 = F::Q1, Q2 = F::Q2, T = kClThreads;
+    constexpr int CA = M / kClCtas, LC = CA + 1, NR = N / kClCtas;   // columns and rows of a CTA
+    static_assert(M % kClCtas == 0 && NR * Q2 <= T && NR * Q1 <= T, "cluster shape");
+    __shared__ float4 Gc[FACET ? 1 : N * CA + N];   // this CTA's cells (and column M in CTA 0)
+    __shared__ float2 Zc[FACET ? 1 : N * LC];       // its columns
+    __shared__ float2 Zr[FACET ? 1 : NR * LD];      // its rows
+    __shared__ float2 tw[FACET ? 1 : N];
+    __shared__ unsigned long long wbest[T / 32];
+    __shared__ float gpos[3];
+    const int c = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nseg = (nl + kClSeg - 1) / kClSeg;
+    const int np = FACET ? nf : N, half = np / 2;             // window size
+    const int rows = (np + kClCtas - 1) / kClCtas;            // window rows of a CTA
+    if (!FACET) {
+        for (int m = tid; m < N; m += T) {
+            float s, cc;
+            sincospif(2.0f * (float)m / (float)N, &s, &cc);
+            tw[m] = make_float2(cc, s);
+        }
+        for (int it = tid; it < N * CA; it += T) Gc[it] = G[(it / CA) * N + c * CA + it % CA];
+        if (c == 0)
+            for (int b = tid; b < N; b += T) Gc[N * CA + b] = G[b * N + M];
+    }
+    int iter = st->iter;
+    const int stop_at = min(max_iter, iter + chunk);
+    bool done = st->done != 0;
+    __syncthreads();
+    while (!done && iter < stop_at) {
+        // peak: every CTA takes the maximum of all row keys
+        unsigned long long k = 0;
+        for (int y = tid; y < nm; y += T) {
+            const unsigned long long q = __ldcg(row + y);
+            k = q > k ? q : k;
+        }
+        k = warp_max(k);
+        if (lane == 0) wbest[warp] = k;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < T / 32; ++w) k = wbest[w] > k ? wbest[w] : k;
+        const int pix = (int)(0xffffffffu - (unsigned int)(k & 0xffffffffull));
+        const unsigned int ob = (unsigned int)(k >> 32);
+        const float peak = __uint_as_float((ob & 0x80000000u) ? (ob & 0x7fffffffu) : ~ob);
+        if (iter > 0 && !(peak > threshold)) {   // the same decision in every thread of the cluster
+            done = true;
+            break;
+        }
+        const int px = pix % nl, py = pix / nl;
+        const float g = gain * peak;
+        float scale;
+        if (FACET) {
+            scale = g / Pf[half * np + half];
+        } else {
+            if (tid == 0) {
+                const double l0 = lc + (px - nl / 2) * cell, m0 = mc + (py - nm / 2) * cell;
+                gpos[0] = literal ? (float)-l0 : (float)m0;
+                gpos[1] = literal ? (float)m0 : (float)-l0;
+                gpos[2] = (float)sqrt(l0 * l0 + m0 * m0);
+            }
+            __syncthreads();
+            const float cx = gpos[0], cb = gpos[1], rho = gpos[2];
+            // (0) X on this CTA's cells (k_img_grid)
+#pragma unroll 4
+            for (int it = tid; it < N * CA; it += T) {
+                const int al = it % CA, b = it / CA, a = c * CA + al;
+                const float4 q = Gc[it];
+                const float af = (float)(a - M), lin0 = af * cx, bf = (float)(b - M);
+                const float sg = ((a + b) & 1) ? -1.f : 1.f;
+                float e = sinc_fast(q.z * fmaf(bf, cb, lin0));
+                if (a == 0 || b == 0) {
+                    const float ma = a == 0 ? af : -af, mb = b == 0 ? bf : -bf;
+                    e = 0.5f * (e + sinc_fast(q.z * fmaf(ma, cx, mb * cb)));
+                }
+                const float d = sg * e * sinc_fast(q.w * rho);
+                Zc[b * LC + al] = make_float2(q.x * d, q.y * d);
+            }
+            if (c == 0)
+                for (int b = tid; b < N; b += T) {
+                    const float4 q = Gc[N * CA + b];
+                    const float bf = (float)(b - M);
+                    float d = sinc_fast(q.z * (bf * cb)) * sinc_fast(q.w * rho);
+                    if ((M + b) & 1) d = -d;
+                    Zc[b * LC + CA] = make_float2(q.x * d, q.y * d);
+                }
+            __syncthreads();
+            // (1a), (1b) columns; the results go to the CTAs that own the rows
+            for (int it = tid; it < CA * R2; it += T) {
+                const int al = it % CA, n2 = it / CA;
+                float2 x[R1];
+#pragma unroll
+                for (int n1 = 0; n1 < R1; ++n1) {
+                    const int r = (n2 + R2 * n1) * LC;
+                    float2 v = Zc[r + al];
+                    if (c == 0 && al == 0) {
+                        const float2 w = Zc[r + CA];
+                        v = make_float2(v.x - w.y, v.y + w.x);
+                    }
+                    x[n1] = v;
+                }
+                dft_reg<R1>(x);
+#pragma unroll
+                for (int k1 = 0; k1 < R1; ++k1) Zc[(n2 + R2 * k1) * LC + al] = cmul(x[k1], tw[n2 * k1]);
+            }
+            __syncthreads();
+            for (int it = tid; it < CA * R1; it += T) {
+                const int al = it % CA, k1 = it / CA, a = c * CA + al;
+                float2 y[R2];
+#pragma unroll
+                for (int n2 = 0; n2 < R2; ++n2) y[n2] = Zc[(R2 * k1 + n2) * LC + al];
+                dft_reg<R2>(y);
+#pragma unroll
+                for (int k2 = 0; k2 < R2; ++k2) {
+                    const int r = k1 + R1 * k2, own = r / NR;
+                    float2 *z = Zr + (r % NR) * LD;
+                    if (a == 0) {
+                        cluster_store(cluster_addr(z, own), make_float2(y[k2].x, 0.f));
+                        cluster_store(cluster_addr(z + M, own), make_float2(y[k2].y, 0.f));
+                    } else {
+                        cluster_store(cluster_addr(z + a, own), y[k2]);
+                    }
+                }
+            }
+            cluster_barrier();
+            // (2a), (2b) rows
+            {
+                float2 v[Q1];
+                const int j = tid % NR, n2 = tid / NR;
+                const bool on = tid < NR * Q2;
+                if (on) {
+#pragma unroll
+                    for (int n1 = 0; n1 < Q1; ++n1) {
+                        const int kk = n2 + Q2 * n1;
+                        const float2 zk = Zr[j * LD + kk], zm = Zr[j * LD + M - kk];
+                        const float2 e = make_float2(zk.x + zm.x, zk.y - zm.y);
+                        const float2 o = cmul(make_float2(zk.x - zm.x, zk.y + zm.y), tw[kk]);
+                        v[n1] = make_float2(e.x - o.y, e.y + o.x);
+                    }
+                }
+                __syncthreads();
+                if (on) {
+                    dft_reg<Q1>(v);
+#pragma unroll
+                    for (int k1 = 0; k1 < Q1; ++k1) Zr[j * LD + n2 + Q2 * k1] = cmul(v[k1], tw[2 * n2 * k1]);
+                }
+            }
+            __syncthreads();
+            {
+                float2 v[Q2];
+                const int j = tid % NR, k1 = tid / NR;
+                const bool on = tid < NR * Q1;
+                if (on) {
+#pragma unroll
+                    for (int n2 = 0; n2 < Q2; ++n2) v[n2] = Zr[j * LD + Q2 * k1 + n2];
+                }
+                __syncthreads();
+                if (on) {
+                    dft_reg<Q2>(v);
+#pragma unroll
+                    for (int k2 = 0; k2 < Q2; ++k2) Zr[j * LD + k1 + Q1 * k2] = v[k2];
+                }
+            }
+            cluster_barrier();
+            // centre pixel (row N/2, sign +)
+            scale = g / cluster_load(cluster_addr(Zr + ((N / 2) % NR) * LD + N / 4, (N / 2) / NR));
+        }
+        // subtract on this CTA's window rows, then renew the rows' maxima
+        const int x0 = max(0, px - half), x1 = min(nl, px - half + np);
+        for (int e = tid; e < rows * np; e += T) {
+            const int jl = e / np, i = e - jl * np, j = c * rows + jl;
+            const int x = px + i - half, y = py + j - half;
+            if (j >= np || x < 0 || x >= nl || y < 0 || y >= nm) continue;
+            float P;
+            if (FACET) {
+                P = Pf[(int64_t)j * np + i];
+            } else {
+                const float2 v = Zr[jl * LD + (i >> 1)];
+                const float sg = (j & 1) ? -1.f : 1.f;
+                P = (i & 1) ? -sg * v.y : sg * v.x;
+            }
+            float *r = res + (int64_t)y * nl + x;
+            *r = __ldcg(r) - scale * P;
+        }
+        if (c == 0 && tid == 0) {
+            if (model) model[pix] += g;
+            if (comp_pix) comp_pix[iter] = pix;
+            if (comp_flux) comp_flux[iter] = g;
+        }
+        __syncthreads();
+        for (int jl = warp; jl < rows; jl += T / 32) {
+            const int j = c * rows + jl, y = py + j - half;
+            if (j < np && y >= 0 && y < nm && x1 > x0)
+                clean_row_keys(res, y, nl, nseg, x0 / kClSeg, (x1 - 1) / kClSeg, seg, row);
+        }
+        ++iter;
+        cluster_barrier();
+    }
+    cluster_barrier();   // no CTA leaves while its shared memory or the record may be read
+    if (c == 0 && tid == 0) {
+        st->iter = iter;
+        st->done = done || iter >= max_iter;
+    }
+}
+
+template <int N, bool FACET>
+cudaError_t launch_clean_loop_t(const float4 *G, const float *P, int nf, float *res, float *model, CleanState *st, int nl,
+                                int nm, double cell, double lc, double mc, float gain, float threshold, int max_iter,
+                                int chunk, int literal, int32_t *cpix, float *cflux, unsigned long long *seg,
+                                unsigned long long *row, cudaStream_t s) {
+    k_clean_loop<N, FACET><<<kClCtas, kClThreads, 0, s>>>(G, P, nf, res, model, st, nl, nm, cell, lc, mc, gain, threshold,
+                                                          max_iter, chunk, literal, cpix, cflux, seg, row);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 bool img_grid_supported(int N) { return N == 16 || N == 32 || N == 64 || N == 128; }
@@ -518,6 +817,35 @@ cudaError_t launch_grid_table(const double2 *S, const double *acc, const double 
     const int64_t n = (int64_t)N * N;
     k_grid_table<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(S, acc, glob, N, du, G);
     return cudaGetLastError();
+}
+
+size_t clean_keys_bytes(int nl, int nm) {
+    return ((size_t)nm * ((nl + kClSeg - 1) / kClSeg) + nm) * sizeof(unsigned long long);
+}
+
+cudaError_t launch_clean_keys(const float *res, int nl, int nm, void *keys, int nsm, cudaStream_t s) {
+    const int nseg = (nl + kClSeg - 1) / kClSeg;
+    unsigned long long *row = (unsigned long long *)keys, *seg = row + nm;
+    k_clean_keys<<<std::min((nm + 7) / 8, 8 * nsm), 256, 0, s>>>(res, nl, nm, nseg, seg, row);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_clean_loop(const float4 *G, const float *P, int N, float *res, float *model, CleanState *st, int nl,
+                              int nm, double cell, double lc, double mc, float gain, float threshold, int max_iter,
+                              int chunk, int literal, int32_t *cpix, float *cflux, void *keys, cudaStream_t s) {
+    unsigned long long *row = (unsigned long long *)keys, *seg = row + nm;
+#define PSF_CLEAN_LOOP(NN, FACET)                                                                                      \
+    return launch_clean_loop_t<NN, FACET>(G, P, N, res, model, st, nl, nm, cell, lc, mc, gain, threshold, max_iter, chunk, \
+                                          literal, cpix, cflux, seg, row, s)
+    if (P) PSF_CLEAN_LOOP(16, true);
+    switch (N) {
+        case 16: PSF_CLEAN_LOOP(16, false);
+        case 32: PSF_CLEAN_LOOP(32, false);
+        case 64: PSF_CLEAN_LOOP(64, false);
+        case 128: PSF_CLEAN_LOOP(128, false);
+        default: return cudaErrorInvalidValue;
+    }
+#undef PSF_CLEAN_LOOP
 }
 
 cudaError_t launch_img_grid(const float4 *G, const GridPos *pos, int npos, int N, float *out, int nsm,

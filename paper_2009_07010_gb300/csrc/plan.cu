@@ -1290,9 +1290,9 @@ int run_img_grid(psf_plan_s *p, const psf_batch_t *b, float *out, cudaStream_t s
     return PSF_OK;
 }
 
-// Hogbom CLEAN with position-dependent PSFs (Algorithm 2).  With the gridded PSF every
-// step of an iteration is a kernel reading the device loop record (k_clean.cu), queued in
-// chunks; the other methods read the peak record back to place the cutout.
+// Hogbom CLEAN with position-dependent PSFs (Algorithm 2).  With the gridded PSF, or one PSF
+// for the whole image, the loop runs inside a kernel (k_clean_loop), many iterations per
+// launch; the other methods read the peak record back to place the cutout (k_clean.cu).
 int run_clean(psf_plan_s *p, const psf_clean_t *c, float *res, float *model, int32_t *cpix, float *cflux,
               int32_t *niter_out, cudaStream_t st) {
     if (!c || !res) return PSF_EINVAL;
@@ -1339,60 +1339,19 @@ int run_clean(psf_plan_s *p, const psf_clean_t *c, float *res, float *model, int
             int s = grid_tables(p, N, c->cell_rad, st, &G);
             if (s) return s;
         }
-        // one chunk of kChunk iterations; kChunk is even, so the alternating argmax keys
-        // repeat identically in every chunk
-        constexpr int kChunk = 64;
-        const int per_iter = facet ? 3 : 4;
-        auto chunk = [&](cudaStream_t cs) -> cudaError_t {
-            for (int q = 0; q < kChunk; ++q) {
-                cudaError_t e = launch_clean_argmax(res, npx, sd, key + (q & 1), p->nsm, cs);
-                if (e == cudaSuccess)
-                    e = launch_clean_prep(key + (q & 1), key + ((q + 1) & 1), sd, c->nl, c->nm, c->cell_rad, c->l_c,
-                                          c->m_c, c->threshold, c->max_iter, literal, cs);
-                if (e == cudaSuccess && !facet) e = launch_img_grid(G, &sd->gpos, 1, N, (float *)P.p, p->nsm, cs);
-                if (e == cudaSuccess)
-                    e = launch_clean_sub(res, model, (const float *)P.p, sd, c->nl, c->nm, N, c->gain, cpix, cflux,
-                                         cs);
-                if (e != cudaSuccess) return e;
-            }
-            return cudaSuccess;
-        };
-        // the first chunk on the caller's stream (it also sets the kernels' one-time
-        // attributes); the loop record is read once per chunk
-        PSF_TRY(chunk(st));
-        if (p->prof) p->n_kernels += per_iter * kChunk;
-        PSF_TRY(cudaMemcpyAsync(&h, sd, sizeof(h), cudaMemcpyDeviceToHost, st));
-        PSF_TRY(cudaStreamSynchronize(st));
-        if (!h.done) {
-            // later chunks: the same launches captured once into a CUDA graph and replayed on
-            // a private stream (the caller's stream has drained; the call returns after the
-            // private stream does)
-            cudaStream_t cs = nullptr;
-            cudaGraph_t g = nullptr;
-            cudaGraphExec_t ge = nullptr;
-            cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-            if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed);
-            if (e == cudaSuccess) {
-                const cudaError_t ec = chunk(cs);
-                e = cudaStreamEndCapture(cs, &g);
-                if (ec != cudaSuccess) e = ec;
-            }
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
-            while (e == cudaSuccess) {
-                e = cudaGraphLaunch(ge, cs);
-                if (e == cudaSuccess) e = cudaMemcpyAsync(&h, sd, sizeof(h), cudaMemcpyDeviceToHost, cs);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
-                if (p->prof) p->n_kernels += per_iter * kChunk;
-                if (e == cudaSuccess && h.done) break;
-            }
-            if (ge) cudaGraphExecDestroy(ge);
-            if (g) cudaGraphDestroy(g);
-            if (cs) cudaStreamDestroy(cs);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                return cuda_status(e);
-            }
-        }
+        // kChunk iterations per launch (a few milliseconds); the loop record is read after each
+        constexpr int kChunk = 1024;
+        DevBuf keys;
+        PSF_TRY(keys.reserve(clean_keys_bytes(c->nl, c->nm)));
+        PSF_TRY(launch_clean_keys(res, c->nl, c->nm, keys.p, p->nsm, st));
+        do {
+            PSF_TRY(launch_clean_loop(G, facet ? (const float *)P.p : nullptr, N, res, model, sd, c->nl, c->nm,
+                                      c->cell_rad, c->l_c, c->m_c, c->gain, c->threshold, c->max_iter, kChunk, literal, cpix,
+                                      cflux, keys.p, st));
+            if (p->prof) p->n_kernels++;
+            PSF_TRY(cudaMemcpyAsync(&h, sd, sizeof(h), cudaMemcpyDeviceToHost, st));
+            PSF_TRY(cudaStreamSynchronize(st));
+        } while (!h.done);
     } else {
         double lm[2] = {0.0, 0.0};
         psf_batch_t b{};
@@ -1402,8 +1361,7 @@ int run_clean(psf_plan_s *p, const psf_clean_t *c, float *res, float *model, int
         b.cell_rad = c->cell_rad;
         for (;; ++t) {
             PSF_TRY(launch_clean_argmax(res, npx, sd, key + (t & 1), p->nsm, st));
-            PSF_TRY(launch_clean_prep(key + (t & 1), key + ((t + 1) & 1), sd, c->nl, c->nm, c->cell_rad,
-                                      c->l_c, c->m_c, c->threshold, c->max_iter, literal, st));
+            PSF_TRY(launch_clean_prep(key + (t & 1), key + ((t + 1) & 1), sd, c->threshold, c->max_iter, st));
             if (p->prof) p->n_kernels += 2;
             PSF_TRY(cudaMemcpyAsync(&h, sd, sizeof(h), cudaMemcpyDeviceToHost, st));
             PSF_TRY(cudaStreamSynchronize(st));

@@ -204,7 +204,6 @@ cudaError_t launch_img_grid(const float4 *G, const GridPos *pos, int npos, int N
 // ---- Hogbom CLEAN (k_clean.cu) ------------------------------------------------
 // Device record of the CLEAN loop (one per call).
 struct CleanState {
-    GridPos gpos;     // position record of the gridded PSF at the current peak (offset 0)
     int32_t done;     // 1 once the loop has stopped
     int32_t iter;     // iterations performed
     int32_t active;   // the current iteration subtracts
@@ -215,11 +214,19 @@ struct CleanState {
 
 cudaError_t launch_clean_argmax(const float *res, int64_t n, const CleanState *st, unsigned long long *key, int nsm,
                                 cudaStream_t s);
-cudaError_t launch_clean_prep(const unsigned long long *key, unsigned long long *key_next, CleanState *st, int nl,
-                              int nm, double cell, double lc, double mc, float threshold, int max_iter, int literal,
-                              cudaStream_t s);
+cudaError_t launch_clean_prep(const unsigned long long *key, unsigned long long *key_next, CleanState *st,
+                              float threshold, int max_iter, cudaStream_t s);
 cudaError_t launch_clean_sub(float *res, float *model, const float *P, CleanState *st, int nl, int nm, int N,
                              float gain, int32_t *comp_pix, float *comp_flux, cudaStream_t s);
+
+// The whole loop on one cluster (k_grid.cu): the gridded PSF at each peak (G, the table of size
+// N) or one given N x N PSF (P).  keys: clean_keys_bytes of device memory, filled by
+// launch_clean_keys from the residual; at most `chunk` iterations per launch.
+size_t clean_keys_bytes(int nl, int nm);
+cudaError_t launch_clean_keys(const float *res, int nl, int nm, void *keys, int nsm, cudaStream_t s);
+cudaError_t launch_clean_loop(const float4 *G, const float *P, int N, float *res, float *model, CleanState *st, int nl,
+                              int nm, double cell, double lc, double mc, float gain, float threshold, int max_iter,
+                              int chunk, int literal, int32_t *cpix, float *cflux, void *keys, cudaStream_t s);
 
 // ---- FWHM along radial / tangential directions (k_fwhm.cu) --------------------
 struct FwhmItem {
