@@ -103,6 +103,58 @@ __device__ __forceinline__ float dirichlet_fast(int F, float a) {
     return sgn * __fdividef(sinpi_fast(Ff * r), Ff * __sinf(x));
 }
 
+// sinc_pi without the special-function and conversion units (each a quarter of the FP32
+// rate or less; with two sines, two quotients and two roundings per weight they bounded
+// the 16-bit weight kernels): sinc_pi(x) = (-1)^n [sin(pi f) / (pi f)] (f / x), x = n + f,
+// |f| <= 1/2, the bracket as its Taylor series to order 10 (truncation error < 4e-8), n by
+// adding 1.5 * 2^23, whose lowest bit is n's parity.  Beyond 4e6 (value below 1e-7): 0.
+__device__ __forceinline__ float sincpi_poly(float x) {
+    const float t = __fadd_rn(x, 12582912.0f);
+    const float n = __fadd_rn(t, -12582912.0f);
+    const float f = x - n;
+    const float z = f * f;
+    float q = fmaf(z, -2.3460810e-3f, 2.6147848e-2f);
+    q = fmaf(z, q, -1.9075182e-1f);
+    q = fmaf(z, q, 8.1174243e-1f);
+    q = fmaf(z, q, -1.6449341f);
+    q = fmaf(z, q, 1.0f);
+    if (n != 0.0f) {
+        q *= __fdividef(f, x);
+        q = fabsf(x) < 4.0e6f ? __int_as_float(__float_as_int(q) ^ (__float_as_int(t) << 31)) : 0.0f;
+    }
+    return q;
+}
+// The Dirichlet kernel as dirichlet_fast, n and its parity by the same addition.
+__device__ __forceinline__ float dirichlet_poly(int F, float a) {
+    const float t = __fadd_rn(a, 12582912.0f);
+    const float r = a - __fadd_rn(t, -12582912.0f);
+    const unsigned sgn = (F & 1) ? 0u : ((unsigned)__float_as_int(t) << 31);
+    const float Ff = (float)F, x = kPiF * r, Fr = Ff * r;
+    float v;
+    if (fabsf(Ff * x) < 0.1f) {
+        const float x2 = x * x, F2 = Ff * Ff;
+        v = 1.0f + x2 * ((1.0f - F2) / 6.0f + x2 * (7.0f / 360.0f - F2 / 36.0f + F2 * F2 / 120.0f));
+    } else {   // sin(pi F r): whole pairs of half turns off
+        const float m = __fadd_rn(__fadd_rn(0.5f * Fr, 12582912.0f), -12582912.0f);
+        v = __fdividef(__sinf(kPiF * (Fr - 2.0f * m)), Ff * __sinf(x));
+    }
+    return __int_as_float(__float_as_int(v) ^ (int)sgn);
+}
+// cos, sin of 2 pi x: MUFU after the same reduction; a series for small steps.
+__device__ __forceinline__ void cis_mufu(float x, float *s, float *c) {
+    const float r = x - __fadd_rn(__fadd_rn(x, 12582912.0f), -12582912.0f);
+    __sincosf(2.0f * kPiF * r, s, c);
+}
+__device__ __forceinline__ void cis_small(float x, float *s, float *c) {
+    if (fabsf(x) < 0.04f) {   // truncation below 2e-8
+        const float y = 2.0f * kPiF * x, y2 = y * y;
+        *s = y * fmaf(y2, fmaf(y2, 1.0f / 120.0f, -1.0f / 6.0f), 1.0f);
+        *c = fmaf(y2, fmaf(y2, fmaf(y2, -1.0f / 720.0f, 1.0f / 24.0f), -0.5f), 1.0f);
+    } else {
+        cis_mufu(x, s, c);
+    }
+}
+
 // Uniform dispatch between the accurate and the fast forms.
 template <bool FAST>
 __device__ __forceinline__ float sincpi_t(float y) { return FAST ? sincpi_fast(y) : sincpi(y); }
