@@ -8,7 +8,9 @@
 // The pixel offsets dl_i, dm_j do not depend on l0 (the cutout moves with the
 // source), so l0 enters through D_k alone.
 //
-// A CTA owns a contiguous range of visibilities; each thread owns kAdjT of them.
+// A CTA owns a contiguous range of visibilities; each thread owns T of them: four, or as
+// few as one where four would leave the chip without enough CTAs (4 positions of 48 pixels on
+// 172 800 visibilities: 425 us with 169 CTAs of four per thread, 304 us with 675 of one).
 // For every position and every 32-row block of R (staged transposed in shared
 // memory) a thread forms t_j = sum_i R[j][i] a_k[i] for the 32 rows (row twiddles by
 // complex recurrence, re-seeded every 32 columns from float-float phases), then adds
@@ -23,7 +25,6 @@ namespace psf {
 namespace {
 
 constexpr int kAdjThreads = 256;
-constexpr int kAdjT = 4;        // visibilities per thread
 constexpr int kAdjRows = 32;    // rows of R per shared-memory block
 constexpr int kAdjMaxN = 512;
 
@@ -35,6 +36,7 @@ struct AdjPos {
     float4 L, dLl, dLm;   // direction (l0, m0, n0-1) and its derivatives
 };
 
+template <int kAdjT>
 __global__ void __launch_bounds__(kAdjThreads) k_adjoint(DevObs o, int method, uint32_t flags,
                                                          const AdjPos *__restrict__ pos,
                                                          const int32_t *__restrict__ npix,
@@ -153,19 +155,40 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint(DevObs o, int method, u
     }
 }
 
+// One warp per element: lane sums over CTAs c = lane (mod 32), then over the lanes, in
+// float64 and in a fixed order.
 __global__ void __launch_bounds__(256) k_adjoint_reduce(const double *__restrict__ partial, int ncta, int npos,
                                                         double *__restrict__ g_lm) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (e >= npos * 2) return;
     double s = 0.0;
-    for (int c = 0; c < ncta; ++c) s += partial[(int64_t)c * npos * 2 + e];
-    g_lm[e] = s;
+    for (int c = lane; c < ncta; c += 32) s += partial[(int64_t)c * npos * 2 + e];
+#pragma unroll
+    for (int sh = 16; sh > 0; sh >>= 1) s += __shfl_down_sync(0xffffffffu, s, sh);
+    if (lane == 0) g_lm[e] = s;
 }
 
 }  // namespace
 
 int adjoint_max_n() { return kAdjMaxN; }
-int64_t adjoint_ctas(int64_t nvis) { return (nvis + kAdjThreads * kAdjT - 1) / (kAdjThreads * kAdjT); }
+static int adjoint_per_thread(int64_t nvis) {   // visibilities per thread: at least ~600 CTAs if possible
+    return nvis >= (int64_t)600 * kAdjThreads * 4 ? 4 : nvis >= (int64_t)600 * kAdjThreads * 2 ? 2 : 1;
+}
+int64_t adjoint_ctas(int64_t nvis) {
+    const int64_t per = (int64_t)kAdjThreads * adjoint_per_thread(nvis);
+    return (nvis + per - 1) / per;
+}
+
+template <int T>
+static cudaError_t launch_adjoint_t(const DevObs &o, int method, uint32_t flags, const void *pos, const int32_t *npix,
+                                    const int64_t *offs, int npos, size_t smem, double cell, const float *R, float *gW,
+                                    int accumulate_gW, double *partial, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(k_adjoint<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_adjoint<T><<<(unsigned)adjoint_ctas(o.nvis), kAdjThreads, smem, st>>>(
+        o, method, flags, (const AdjPos *)pos, npix, offs, npos, fp32t::cell_pair(cell), R, gW, accumulate_gW, partial);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_adjoint_chunk(const DevObs &o, int method, uint32_t flags, const void *pos, const int32_t *npix,
                                  const int64_t *offs, int npos, int nmax, double cell, const float *R, float *gW,
@@ -173,13 +196,14 @@ cudaError_t launch_adjoint_chunk(const DevObs &o, int method, uint32_t flags, co
     if (npos <= 0) return cudaSuccess;
     const int64_t ncta = adjoint_ctas(o.nvis);
     const size_t smem = (size_t)nmax * kAdjRows * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e;
+    switch (adjoint_per_thread(o.nvis)) {
+        case 4: e = launch_adjoint_t<4>(o, method, flags, pos, npix, offs, npos, smem, cell, R, gW, accumulate_gW, partial, st); break;
+        case 2: e = launch_adjoint_t<2>(o, method, flags, pos, npix, offs, npos, smem, cell, R, gW, accumulate_gW, partial, st); break;
+        default: e = launch_adjoint_t<1>(o, method, flags, pos, npix, offs, npos, smem, cell, R, gW, accumulate_gW, partial, st);
+    }
     if (e != cudaSuccess) return e;
-    k_adjoint<<<(unsigned)ncta, kAdjThreads, smem, st>>>(o, method, flags, (const AdjPos *)pos, npix, offs, npos,
-                                                         fp32t::cell_pair(cell), R, gW, accumulate_gW, partial);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_adjoint_reduce<<<(npos * 2 + 255) / 256, 256, 0, st>>>(partial, (int)ncta, npos, g_lm);
+    k_adjoint_reduce<<<(npos * 2 + 7) / 8, 256, 0, st>>>(partial, (int)ncta, npos, g_lm);
     return cudaGetLastError();
 }
 
