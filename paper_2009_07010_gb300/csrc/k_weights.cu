@@ -157,11 +157,13 @@ __global__ void __launch_bounds__(256) k_weights_exact8(DevObs o, const float4 *
 // consecutive channels of one bin.  Per bin the frequency sinc is the same for every channel
 // (Method 1: ubar . L Dnu / c; Method 2: (Dnu / nu) |u| |l0| = |ubar| Dnu / c |l0|, with equal
 // Dnu), and the time sinc's argument is linear in nu_r.  One visibility per thread, each with
-// its own integer division, records and two MUFU sincs, took 376 us for 58.1 M visibilities;
-// now 200 us.
-__global__ void __launch_bounds__(256) k_weights_real8(DevObs o, int method, uint32_t flags,
-                                                       const float4 *__restrict__ pos, int32_t k0, int32_t kn,
-                                                       float2 *__restrict__ w, int64_t ldw) {
+// its own integer division, records and two MUFU sincs, took 376 us per method for 58.1 M
+// visibilities; now 200 us, and 319 us for both methods in one pass (METHODS bit 0: Method 1
+// into w, bit 1: Method 2 into w2).
+template <int METHODS>
+__global__ void __launch_bounds__(256) k_weights_real8(DevObs o, uint32_t flags, const float4 *__restrict__ pos,
+                                                       int32_t k0, int32_t kn, float2 *__restrict__ w,
+                                                       float2 *__restrict__ w2, int64_t ldw) {
     const int p = blockIdx.y;
     const float4 L = pos[p];
     const float rho = sqrtf(L.x * L.x + L.y * L.y);
@@ -169,56 +171,86 @@ __global__ void __launch_bounds__(256) k_weights_real8(DevObs o, int method, uin
         const int32_t kk0 = 8 * g, kb = k0 + kk0;
         const int bin = kb / o.nout, r0 = kb - bin * o.nout;
         const float4 ub = o.bin_ubar[bin], ch = o.chan[r0];
-        float a, B;   // time sinc argument per frequency, frequency sinc argument
-        if (method == kUV) {
-            a = dot3(o.bin_edge[bin], L) * kInvC;
-            B = dot3(ub, L) * ch.y * kInvC;
-        } else {
-            const float len = sqrtf(ub.x * ub.x + ub.y * ub.y);
-            float udot = -ub.y, vdot = ub.x;
-            if (flags & PSF_IMG_LITERAL_THETA) {
-                const float th = (ub.y != 0.0f) ? atanf(ub.x / ub.y) : (ub.x >= 0.0f ? 0.5f * kPiF : -0.5f * kPiF);
-                float st, ct;
-                sincosf(th, &st, &ct);
-                udot = -len * st;
-                vdot = len * ct;
-            }
-            a = (float)kOmegaE * ub.w * (udot * L.x + vdot * L.y) * kInvC;
-            B = ch.y * kInvC * len * rho;
-        }
-        const float sB = sincpi_poly(B);
-        float2 *dst = w + (int64_t)p * ldw + kk0;
+        float Wk[8];
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-            const float v0 = sB * sincpi_poly(a * fmaf((float)j, o.dnu_ch, ch.x));
-            const float v1 = sB * sincpi_poly(a * fmaf((float)(j + 1), o.dnu_ch, ch.x));
-            if (kk0 + j + 1 < kn)   // ldw and kk0 + j are even: 16-byte aligned
-                *reinterpret_cast<float4 *>(dst + j) = make_float4(o.W[kb + j] * v0, 0.f, o.W[kb + j + 1] * v1, 0.f);
-            else if (kk0 + j < kn)
-                dst[j] = make_float2(o.W[kb + j] * v0, 0.f);
+        for (int j = 0; j < 8; ++j) Wk[j] = kk0 + j < kn ? o.W[kb + j] : 0.f;
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            if (!(METHODS & (1 << m))) continue;
+            float a, B;   // time sinc argument per frequency, frequency sinc argument
+            if (m == 0) {
+                a = dot3(o.bin_edge[bin], L) * kInvC;
+                B = dot3(ub, L) * ch.y * kInvC;
+            } else {
+                const float len = sqrtf(ub.x * ub.x + ub.y * ub.y);
+                float udot = -ub.y, vdot = ub.x;
+                if (flags & PSF_IMG_LITERAL_THETA) {
+                    const float th = (ub.y != 0.0f) ? atanf(ub.x / ub.y) : (ub.x >= 0.0f ? 0.5f * kPiF : -0.5f * kPiF);
+                    float st, ct;
+                    sincosf(th, &st, &ct);
+                    udot = -len * st;
+                    vdot = len * ct;
+                }
+                a = (float)kOmegaE * ub.w * (udot * L.x + vdot * L.y) * kInvC;
+                B = ch.y * kInvC * len * rho;
+            }
+            const float sB = sincpi_poly(B);
+            float2 *dst = (m == 0 ? w : w2) + (int64_t)p * ldw + kk0;
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                const float v0 = Wk[j] * sB * sincpi_poly(a * fmaf((float)j, o.dnu_ch, ch.x));
+                const float v1 = Wk[j + 1] * sB * sincpi_poly(a * fmaf((float)(j + 1), o.dnu_ch, ch.x));
+                if (kk0 + j + 1 < kn)   // ldw and kk0 + j are even: 16-byte aligned
+                    *reinterpret_cast<float4 *>(dst + j) = make_float4(v0, 0.f, v1, 0.f);
+                else if (kk0 + j < kn)
+                    dst[j] = make_float2(v0, 0.f);
+            }
         }
     }
+}
+
+// Channels shared by eight-channel groups aligned with the range.
+static bool groups_of_8(const DevObs &o, int32_t k0) { return o.chan_affine && o.nout % 8 == 0 && k0 % 8 == 0; }
+
+static int weight_sms() {   // SM count of the first device used (only sizes the grids)
+    static int nsm = 0;
+    if (nsm == 0 && cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, 0) != cudaSuccess) {
+        cudaGetLastError();
+        nsm = 152;
+    }
+    return nsm;
+}
+static dim3 grid_of_8(int32_t kn, int npos) {
+    const int64_t b = std::min<int64_t>((kn / 8 + 255) / 256 + 1,
+                                        (int64_t)weight_sms() * 16 / std::max(1, std::min(npos, 16)));
+    return dim3((unsigned)std::max<int64_t>(1, b), npos);
+}
+
+cudaError_t launch_weights_uvimg(const DevObs &o, uint32_t flags, const float4 *pos, int npos, int32_t nvis,
+                                 float2 *w_uv, float2 *w_img, int64_t ldw, int *nkernels, cudaStream_t st) {
+    *nkernels = 0;
+    if (npos <= 0 || nvis <= 0) return cudaSuccess;
+    if (!o.win && groups_of_8(o, 0)) {
+        *nkernels = 1;
+        k_weights_real8<3><<<grid_of_8(nvis, npos), 256, 0, st>>>(o, flags, pos, 0, nvis, w_uv, w_img, ldw);
+        return cudaGetLastError();
+    }
+    *nkernels = 2;
+    const cudaError_t e = launch_weights(o, kUV, flags, pos, npos, 0, nvis, w_uv, ldw, 1, st);
+    return e != cudaSuccess ? e : launch_weights(o, kImg, flags, pos, npos, 0, nvis, w_img, ldw, 1, st);
 }
 
 cudaError_t launch_weights(const DevObs &o, int method, uint32_t flags, const float4 *pos, int npos,
                            int32_t k0, int32_t kn, float2 *w, int64_t ldw, int fast, cudaStream_t st) {
     if (npos <= 0 || kn <= 0) return cudaSuccess;
-    static int nsm = 0;   // SM count of the first device used (only sizes the grid)
-    if (nsm == 0 && cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, 0) != cudaSuccess) {
-        cudaGetLastError();
-        nsm = 152;
-    }
-    const int64_t blocks = std::min<int64_t>((kn + 255) / 256, (int64_t)nsm * 16 / std::max(1, std::min(npos, 16)));
+    const int64_t blocks =
+        std::min<int64_t>((kn + 255) / 256, (int64_t)weight_sms() * 16 / std::max(1, std::min(npos, 16)));
     dim3 grid((unsigned)std::max<int64_t>(1, blocks), npos);
-    if (fast && method == kExact && o.chan_affine && o.nout % 8 == 0 && k0 % 8 == 0) {
-        const int64_t b8 = std::min<int64_t>((kn / 8 + 255) / 256 + 1, (int64_t)nsm * 16 / std::max(1, std::min(npos, 16)));
-        k_weights_exact8<<<dim3((unsigned)std::max<int64_t>(1, b8), npos), 256, 0, st>>>(o, pos, k0, kn, w, ldw);
-        return cudaGetLastError();
-    }
-    if (fast && method != kExact && !o.win && o.chan_affine && o.nout % 8 == 0 && k0 % 8 == 0) {
-        const int64_t b8 = std::min<int64_t>((kn / 8 + 255) / 256 + 1, (int64_t)nsm * 16 / std::max(1, std::min(npos, 16)));
-        k_weights_real8<<<dim3((unsigned)std::max<int64_t>(1, b8), npos), 256, 0, st>>>(o, method, flags, pos, k0, kn, w,
-                                                                                       ldw);
+    if (fast && !o.win && groups_of_8(o, k0)) {
+        const dim3 g8 = grid_of_8(kn, npos);
+        if (method == kExact) k_weights_exact8<<<g8, 256, 0, st>>>(o, pos, k0, kn, w, ldw);
+        else if (method == kUV) k_weights_real8<1><<<g8, 256, 0, st>>>(o, flags, pos, k0, kn, w, nullptr, ldw);
+        else k_weights_real8<2><<<g8, 256, 0, st>>>(o, flags, pos, k0, kn, nullptr, w, ldw);
         return cudaGetLastError();
     }
     if (fast) k_weights<true><<<grid, 256, 0, st>>>(o, method, flags, pos, k0, kn, w, ldw);
@@ -663,7 +695,12 @@ __global__ void __launch_bounds__(256) k_reduce(const float *__restrict__ partia
                                                 int64_t stride, const int64_t *__restrict__ loc_offs,
                                                 const int64_t *__restrict__ out_offs,
                                                 const int32_t *__restrict__ npix, int transposed,
-                                                float *__restrict__ out) {
+                                                float *__restrict__ out, const float *__restrict__ partial2,
+                                                float *__restrict__ out2) {
+    if (blockIdx.z) {
+        partial = partial2;
+        out = out2;
+    }
     __shared__ double sum[8][32];
     const int p = blockIdx.y;
     const int N = npix[p];
@@ -700,10 +737,10 @@ __global__ void __launch_bounds__(256) k_reduce(const float *__restrict__ partia
 
 cudaError_t launch_reduce(const float *partial, int nsplit, int64_t stride, const int64_t *loc_offs,
                           const int64_t *out_offs, const int32_t *npix, int npos, int transposed, float *out,
-                          cudaStream_t st) {
+                          cudaStream_t st, const float *partial2, float *out2) {
     if (npos <= 0) return cudaSuccess;
-    dim3 grid((unsigned)std::max(16, 512 / npos), npos);
-    k_reduce<<<grid, 256, 0, st>>>(partial, nsplit, stride, loc_offs, out_offs, npix, transposed, out);
+    dim3 grid((unsigned)std::max(16, 512 / npos), npos, partial2 ? 2 : 1);
+    k_reduce<<<grid, 256, 0, st>>>(partial, nsplit, stride, loc_offs, out_offs, npix, transposed, out, partial2, out2);
     return cudaGetLastError();
 }
 

@@ -1068,9 +1068,9 @@ int run_forward_uvimg(psf_plan_s *p, const psf_batch_t *b, float *out_uv, float 
         const int64_t wblock = cn * ldw + 64;
         PSF_TRY(p->wbuf.reserve((size_t)(2 * wblock) * sizeof(float2)));
         float2 *w_uv = (float2 *)p->wbuf.p, *w_img = w_uv + wblock;
-        PSF_TRY(launch_weights(p->d, kUV, p->opts.flags, d_pos, cn, 0, (int32_t)K, w_uv, ldw, 1, st));
-        PSF_TRY(launch_weights(p->d, kImg, p->opts.flags, d_pos, cn, 0, (int32_t)K, w_img, ldw, 1, st));
-        p->n_kernels += 2;
+        int nw = 0;
+        PSF_TRY(launch_weights_uvimg(p->d, p->opts.flags, d_pos, cn, (int32_t)K, w_uv, w_img, ldw, &nw, st));
+        p->n_kernels += nw;
         const int64_t part2 = (int64_t)nsplit * chunk_px;
         PSF_TRY(p->partial.reserve((size_t)(2 * part2) * sizeof(float)));
         float *part = (float *)p->partial.p;
@@ -1093,9 +1093,8 @@ int run_forward_uvimg(psf_plan_s *p, const psf_batch_t *b, float *out_uv, float 
         if (p->prof) PSF_TRY(cudaEventRecord(ev2, st));
         p->n_contract++;
         p->n_kernels++;
-        PSF_TRY(launch_reduce(part, nsplit, chunk_px, d_loc, d_out, d_npix, cn, 1, out_uv, st));
-        PSF_TRY(launch_reduce(part + part2, nsplit, chunk_px, d_loc, d_out, d_npix, cn, 1, out_img, st));
-        p->n_kernels += 2;
+        PSF_TRY(launch_reduce(part, nsplit, chunk_px, d_loc, d_out, d_npix, cn, 1, out_uv, st, part + part2, out_img));
+        p->n_kernels++;
     }
     return PSF_OK;
 }

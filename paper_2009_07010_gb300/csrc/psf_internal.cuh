@@ -60,6 +60,10 @@ enum Method { kExact = 0, kUV = 1, kImg = 2 };
 cudaError_t launch_weights(const DevObs &o, int method, uint32_t flags, const float4 *pos,
                            int npos, int32_t k0, int32_t kn, float2 *w, int64_t ldw, int fast,
                            cudaStream_t st);
+// Weights of Methods 1 and 2 (no windows) of all nvis visibilities, FAST forms, in one launch
+// where the channels allow it; *nkernels receives the number of launches.
+cudaError_t launch_weights_uvimg(const DevObs &o, uint32_t flags, const float4 *pos, int npos, int32_t nvis,
+                                 float2 *w_uv, float2 *w_img, int64_t ldw, int *nkernels, cudaStream_t st);
 // FP32 CUDA-core contraction; partial[split * split_stride + out_off + j*N + i].
 cudaError_t launch_psf_fp32(const DevObs &o, const float2 *w, int64_t ldw, const Tile *tiles,
                             int ntiles, int nsplit, int32_t kper, double cell, float *partial,
@@ -68,10 +72,11 @@ cudaError_t launch_psf_fp32(const DevObs &o, const float2 *w, int64_t ldw, const
 // its size in columns and rows.
 int fp32_shape(const int32_t *npix, int npos, int *ti, int *tj);
 // out[out_off_p + q] = sum_s partial[s * stride + loc_off_p + q'] (float64 sum), where
-// q' = q for row-major partials and q' = i N + j for q = j N + i when `transposed`.
+// q' = q for row-major partials and q' = i N + j for q = j N + i when `transposed`;
+// partial2, out2: a second set of the same layout in the same launch.
 cudaError_t launch_reduce(const float *partial, int nsplit, int64_t stride, const int64_t *loc_offs,
                           const int64_t *out_offs, const int32_t *npix, int npos, int transposed, float *out,
-                          cudaStream_t st);
+                          cudaStream_t st, const float *partial2 = nullptr, float *out2 = nullptr);
 // Plan-time per-visibility tables: uv[k] + uv_lo[k] (from the float64 bin means and
 // channel frequencies) and, if natural, W[k] = tavg * favg.
 // Averaging bins of the plan from the raw uvw on the device (k_weights.cu, k_bin).
