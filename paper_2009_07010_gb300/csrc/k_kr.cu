@@ -61,6 +61,7 @@ constexpr int kKrTmaWarp = 20;
 constexpr int kKrMmaWarp = 21;
 constexpr int kKrInWarp = 22;
 constexpr int kKrThreads = 23 * 32;
+constexpr int kKrAhead = 12;          // stages between an L2 prefetch and its copy
 constexpr uint32_t kKrATile = 128 * 128;   // 128 positions x 64 visibilities x 2 B
 constexpr uint32_t kKrBTile = 256 * 128;   // 256 twiddle rows x 64 visibilities x 2 B
 constexpr uint32_t kKrInSlot = kKrKS * 8;  // uv per stage
@@ -371,6 +372,10 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                     if (used) phase_bits ^= 1u << slot;
                     used_bits |= 1u << slot;
                     mbar_arrive_expect_tx(&full[slot], Sh::kA);
+                    // With complex weights (three slots, twice the bytes) the copies' latency shows: one CTA
+                    // per tile row brings later stages into L2 (contraction of 256 x 64^2 exact 22.6 ->
+                    // 21.7 ms; with real weights 57.5 -> 61 ms, so not there).
+                    if (!REAL && it.q0 == 0 && s + kKrAhead < nst) bulk_prefetch_l2(src + (int64_t)(s + kKrAhead) * Sh::kA, Sh::kA);
                     bulk_g2s(a_base + slot * Sh::kA, src + (int64_t)s * Sh::kA, Sh::kA, &full[slot]);
                 }
                 if (stop) break;

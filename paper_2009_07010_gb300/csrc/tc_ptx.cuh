@@ -99,6 +99,11 @@ static __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint
         : "memory");
 }
 
+// The same bytes into L2 only.
+static __device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 static __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
