@@ -735,8 +735,8 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
 // Autotuner of the batched form, run on the first batched call of a plan for each weight
 // class (real / complex weights, operand type) and cutout size N and cached in the plan: the
 // crossover between the forms.  Over a probe of the first kProbeVis visibilities it times
-// the per-cutout form for one position and the batched form for one 128-position tile; the
-// batched form takes a group of n positions when ceil(n / 128) t_tile < n t_cutout.
+// the per-cutout form for one more position and the batched form for one 128-position tile;
+// the batched form takes whole tiles, and a remainder of n positions when t_tile < n t_cutout.
 constexpr int64_t kProbeVis = int64_t(1) << 19;
 
 int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cudaStream_t st, int64_t kmax = -1);
@@ -767,27 +767,37 @@ int kr_tune(psf_plan_s *p, int method, const BatchHost &hall, const std::vector<
         one[0].idx.assign(g.idx.begin(), g.idx.begin() + std::min<size_t>(g.idx.size(), 128));
         double t_tile = 0.0;
         if ((s = run_kr(p, method, hs, one, (float *)scratch.p, st, probe, &t_tile))) break;
-        const double lm[2] = {0.0, 0.0};   // cost does not depend on the position
+        // one more cutout in the per-cutout form: the difference of five and one, so that neither
+        // launches nor the probe's short range count (with the time of a single cutout a tile was
+        // taken for 14 positions of 128 pixels, whose 33 of 217 tile columns cost 8 ms where 14
+        // cutouts cost 4)
+        const double lm[10] = {};   // cost does not depend on the position
         psf_batch_t b1{};
-        b1.npos = 1;
         b1.lm = lm;
         b1.npix0 = g.N;
         b1.cell_rad = hall.cell;
+        DevBuf cut;
+        PSF_TRY(cut.reserve((size_t)5 * g.N * g.N * sizeof(float)));
         const psf_opts_t saved = p->opts;
         p->opts.algo = PSF_ALGO_CUTOUT;
-        cudaEvent_t a, z;
-        PSF_TRY(cudaEventCreate(&a));
-        PSF_TRY(cudaEventCreate(&z));
-        PSF_TRY(cudaEventRecord(a, st));
-        s = run_forward(p, method, &b1, (float *)scratch.p, st, probe);
-        PSF_TRY(cudaEventRecord(z, st));
-        PSF_TRY(cudaEventSynchronize(z));
-        float t_cut = 0.f;
-        PSF_TRY(cudaEventElapsedTime(&t_cut, a, z));
-        cudaEventDestroy(a);
-        cudaEventDestroy(z);
+        cudaEvent_t ev[3] = {};
+        for (auto &e : ev) PSF_TRY(cudaEventCreate(&e));
+        b1.npos = 5;
+        s = run_forward(p, method, &b1, (float *)cut.p, st, probe);   // buffers, first launch
+        PSF_TRY(cudaEventRecord(ev[0], st));
+        if (!s) s = run_forward(p, method, &b1, (float *)cut.p, st, probe);
+        PSF_TRY(cudaEventRecord(ev[1], st));
+        b1.npos = 1;
+        if (!s) s = run_forward(p, method, &b1, (float *)cut.p, st, probe);
+        PSF_TRY(cudaEventRecord(ev[2], st));
+        PSF_TRY(cudaEventSynchronize(ev[2]));
+        float t5 = 0.f, t1 = 0.f;
+        PSF_TRY(cudaEventElapsedTime(&t5, ev[0], ev[1]));
+        PSF_TRY(cudaEventElapsedTime(&t1, ev[1], ev[2]));
+        for (auto &e : ev) cudaEventDestroy(e);
         p->opts = saved;
-        const double thr = t_cut > 0.f ? t_tile / (double)t_cut : 1e9;
+        const double t_cut = std::max(0.25 * (t5 - t1), 0.05 * t5);
+        const double thr = t_cut > 0.0 ? t_tile / t_cut : 1e9;
         t.min_group[g.N] = (int)std::max(1.0, std::min(128.0, std::ceil(thr)));
     }
     p->prof = prof;
@@ -834,9 +844,14 @@ int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cud
         for (const auto &g : present) {
             const auto f = t.min_group.find(g.N);
             const int thr = f != t.min_group.end() ? f->second : kKrMinGroup;
-            if ((int)g.idx.size() < thr) continue;
-            batched.push_back(g);
-            for (int i : g.idx) done[i] = 1;
+            // whole 128-position tiles, and a remainder large enough for a tile of its own: 14
+            // positions over 128 cost as much as 128 more (33 of 217 pixel-tile columns of a call of
+            // 512 mixed cutouts)
+            const int n = (int)g.idx.size(), rem = n % 128;
+            const int keep = rem >= thr ? n : n - rem;
+            if (keep == 0) continue;
+            batched.push_back(KrGroup{g.N, std::vector<int>(g.idx.begin(), g.idx.begin() + keep)});
+            for (int i = 0; i < keep; ++i) done[g.idx[i]] = 1;
         }
         if (!batched.empty() && (s = run_kr(p, method, hall, batched, out, st))) return s;
         for (int i = 0; i < hall.npos; ++i)
