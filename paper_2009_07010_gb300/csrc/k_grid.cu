@@ -173,8 +173,13 @@ __global__ void k_grid_table(const double2 *__restrict__ S, const double *__rest
 // sinc_pi(x) = sin(pi x) / (pi x) = (-1)^n [sin(pi f) / (pi f)] (f / x), x = n + f, |f| <= 1/2.
 // n comes from adding 1.5 * 2^23 (|x| < 2^22), which rounds x to the nearest integer and
 // leaves the parity of n in the lowest mantissa bit; the bracket is its Taylor series in
-// (pi f)^2 to order 10 (truncation error < 4e-8).
-__device__ __forceinline__ float sinc_fast(float x) {
+// (pi f)^2 to order 10 (truncation error < 4e-8).  f / x (1 for n = 0) is left as a fraction.
+struct SincParts {
+    float q, num, den;
+    int parity;
+};
+
+__device__ __forceinline__ SincParts sinc_parts(float x) {
     const float t = x + 12582912.0f;
     const float n = t - 12582912.0f;
     const float f = x - n;
@@ -184,8 +189,28 @@ __device__ __forceinline__ float sinc_fast(float x) {
     q = fmaf(z, q, 8.1174243e-1f);
     q = fmaf(z, q, -1.6449341f);
     q = fmaf(z, q, 1.0f);
-    if (n != 0.0f) q *= __fdividef(f, x);
-    return __int_as_float(__float_as_int(q) ^ (__float_as_int(t) << 31));
+    const bool nz = n != 0.0f;
+    return {q, nz ? f : 1.0f, nz ? x : 1.0f, __float_as_int(t)};
+}
+
+// sinc_pi(x) sinc_pi(y) with one quotient.
+__device__ __forceinline__ float sinc2_fast(float x, float y) {
+    const SincParts a = sinc_parts(x), b = sinc_parts(y);
+    const float v = (a.q * b.q) * __fdividef(a.num * b.num, a.den * b.den);
+    return __int_as_float(__float_as_int(v) ^ ((a.parity ^ b.parity) << 31));
+}
+
+// D' of a cell (offsets af, bf from the grid's centre): its smearing factor, averaged with that
+// of the mirror cell modulo N on the Nyquist row and column.
+__device__ __forceinline__ float cell_factor(const float4 &g, float af, float bf, float lin0, float cx, float cb,
+                                             float rho, bool a0, bool b0) {
+    const float y = g.w * rho;
+    float d = sinc2_fast(g.z * fmaf(bf, cb, lin0), y);
+    if (a0 || b0) {
+        const float ma = a0 ? af : -af, mb = b0 ? bf : -bf;
+        d = 0.5f * (d + sinc2_fast(g.z * fmaf(ma, cx, mb * cb), y));
+    }
+    return d;
 }
 
 __host__ __device__ constexpr int ilog2(int r) { return r <= 1 ? 0 : 1 + ilog2(r / 2); }
@@ -249,44 +274,57 @@ __device__ __forceinline__ void dft_reg(float2 (&x)[R]) {
 }
 
 // Shapes: the column transforms (length N over b) run as R1 x R2 Cooley-Tukey, the row
-// transforms (length M = N/2, the complex core of each real row) as Q1 x Q2; T threads;
-// the second stages of both passes take their lines in P parts to bound registers.
+// transforms (length M = N/2, the complex core of each real row) as Q1 x Q2; T threads.
 template <int N>
 struct GridFft;
 template <>
-struct GridFft<16> { static constexpr int R1 = 4, R2 = 4, Q1 = 4, Q2 = 2, T = 64, P = 1; };
+struct GridFft<16> { static constexpr int R1 = 4, R2 = 4, Q1 = 4, Q2 = 2, T = 64; };
 template <>
-struct GridFft<32> { static constexpr int R1 = 8, R2 = 4, Q1 = 4, Q2 = 4, T = 128, P = 1; };
+struct GridFft<32> { static constexpr int R1 = 8, R2 = 4, Q1 = 4, Q2 = 4, T = 128; };
 template <>
-struct GridFft<64> { static constexpr int R1 = 8, R2 = 8, Q1 = 8, Q2 = 4, T = 128, P = 1; };
+struct GridFft<64> { static constexpr int R1 = 8, R2 = 8, Q1 = 8, Q2 = 4, T = 128; };
 template <>
-struct GridFft<128> { static constexpr int R1 = 16, R2 = 8, Q1 = 8, Q2 = 8, T = 256, P = 2; };
+struct GridFft<128> { static constexpr int R1 = 16, R2 = 8, Q1 = 8, Q2 = 8, T = 256; };
+
+// Row stride of Z in k_img_grid: Q2 past the M columns, so that the rows a half warp works on
+// (16 / Q2 of them, Q2 lanes each) fall on different banks.
+template <int N>
+__host__ __device__ constexpr int grid_ld() { return N / 2 + GridFft<N>::Q2; }
 
 template <int N>
-constexpr int grid_smem_bytes() { return (N * (N / 2 + 1) + N) * (int)sizeof(float2); }
+constexpr int grid_smem_bytes() { return (N * grid_ld<N>() + N) * (int)sizeof(float2); }
 
 template <int N>
 constexpr int grid_min_blocks() { return N == 128 ? 3 : N == 64 ? 6 : 8; }
 
 // One CTA per position (grid-stride).  X = (-1)^(a+b) S D' is Hermitian, so only the
-// cells a in [0, N/2] are formed, in shared memory Z [N rows][N/2 + 1] (row b, later
-// output row j; the odd row stride keeps every lane pattern below free of bank
-// conflicts), with the N twiddles exp(+2 pi i m / N).
-//   (0) X on the half grid, flat over its cells
-//   (1) columns: length-N inverse DFT over b for a in [0, N/2); column 0 carries
-//       X[.][0] + i X[.][N/2], whose transforms are both real, and is unpacked into them
+// cells a in [0, N/2] are formed, with the N twiddles exp(+2 pi i m / N) in shared memory.
+// Z [N rows][LD], row b, later output row j, holds what passes between the stages.
+//   (0) the columns a = 0 and a = N/2 of X into Z's columns M and M + 1
+//   (1) columns: length-N inverse DFT over b for a in [0, N/2), the first stage on cells that
+//       the thread forms itself; column 0 carries X[.][0] + i X[.][N/2], whose transforms are
+//       both real, and is unpacked into them
 //   (2) rows: each row j is Hermitian in a, and its real inverse DFT x is obtained from
 //       one length-N/2 complex DFT of C[k] = E[k] + i O[k], E[k] = Z[k] + conj Z[N/2 - k],
-//       O[k] = (Z[k] - conj Z[N/2 - k]) exp(2 pi i k / N): it returns x[2n] + i x[2n+1]
-//   (3) out[j][i] = (-1)^(i + j) x[i], two floats per store.
+//       O[k] = (Z[k] - conj Z[N/2 - k]) exp(2 pi i k / N): it returns x[2n] + i x[2n+1];
+//       out[j][i] = (-1)^(i + j) x[i], two floats per store.
 // Cell and pixel index origins are at N/2: exp(2 pi i (a - N/2)(i - N/2) / N) =
 // (-1)^(a + i) exp(2 pi i a i / N) for N % 4 == 0.
+//
+// Bound by instruction issue (268 MB written for 4096 positions of 128 pixels take 40 us).  With
+// X written to Z before the first stage, block-wide exchanges between all stages and the result
+// once more through Z it took 52.4 k warp instructions per position and 250 us for those; now
+// 43.9 k and 212 us: the first stage works on its own cells, the second stage of the columns
+// in place (stage one stores (n2, k1) as row k1 + R1 n2, from where the thread that takes k1
+// reads and to where it writes), a row stays within one warp, and the two sincs of a cell
+// share a quotient.
 template <int N>
 __global__ void __launch_bounds__(GridFft<N>::T, grid_min_blocks<N>())
     k_img_grid(const float4 *__restrict__ G, const GridPos *__restrict__ pos, int npos, float *__restrict__ out) {
     using F = GridFft<N>;
-    constexpr int M = N / 2, LD = M + 1, T = F::T, R1 = F::R1, R2 = F::R2, Q1 = F::Q1, Q2 = F::Q2, P = F::P;
-    static_assert(R1 * R2 == N && Q1 * Q2 == M && M % P == 0 && N % P == 0, "shape");
+    constexpr int M = N / 2, LD = grid_ld<N>(), T = F::T, R1 = F::R1, R2 = F::R2, Q1 = F::Q1, Q2 = F::Q2;
+    constexpr int RW = 32 / Q2;   // rows of a warp at a time
+    static_assert(R1 * R2 == N && Q1 * Q2 == M && Q1 % Q2 == 0 && R2 % 2 == 0 && N % RW == 0, "shape");
     extern __shared__ float2 smem[];
     float2 *Z = smem;
     float2 *tw = smem + N * LD;
@@ -295,177 +333,111 @@ __global__ void __launch_bounds__(GridFft<N>::T, grid_min_blocks<N>())
         sincospif(2.0f * (float)m / (float)N, &s, &c);
         tw[m] = make_float2(c, s);
     }
-    __syncthreads();
+    const int lane = threadIdx.x & 31;
     for (int p = blockIdx.x; p < npos; p += gridDim.x) {
         const GridPos gp = pos[p];
-        // (0) X = (-1)^(a+b) S D' on the cells a in [0, M]; D' = D except on the Nyquist
-        // row and column, where it is averaged with the mirror cell modulo N.  Columns
-        // a < M: a fixed per thread, rows b0, b0 + RS, ... (RS even: the sign is fixed too);
-        // column M: one row per thread.
-        {
-            constexpr int RS = T / M;
-            static_assert(T % M == 0 && RS % 2 == 0 && T >= N, "pre-pass shape");
-            const int a = threadIdx.x % M, b0 = threadIdx.x / M;
-            const float af = (float)(a - M), lin0 = af * gp.c.x, cb = gp.c.y, rho = gp.c.z;
-            const float sg = ((a + b0) & 1) ? -1.f : 1.f;
-#pragma unroll 4
-            for (int b = b0; b < N; b += RS) {
-                const float4 g = __ldg(G + b * N + a);
-                const float bf = (float)(b - M);
-                float e = sinc_fast(g.z * fmaf(bf, cb, lin0));
-                if (a == 0 || b == 0) {
-                    const float ma = a == 0 ? af : -af, mb = b == 0 ? bf : -bf;
-                    e = 0.5f * (e + sinc_fast(g.z * fmaf(ma, gp.c.x, mb * cb)));
-                }
-                const float d = sg * e * sinc_fast(g.w * rho);
-                Z[b * LD + a] = make_float2(g.x * d, g.y * d);
-            }
-            for (int b = threadIdx.x; b < N; b += T) {
-                const float4 g = __ldg(G + b * N + M);
-                const float bf = (float)(b - M);
-                // a' = 0: the mirror (0, -b') has the same D (D is even), so D' = D here
-                float d = sinc_fast(g.z * (bf * cb)) * sinc_fast(g.w * rho);
-                if ((M + b) & 1) d = -d;
-                Z[b * LD + M] = make_float2(g.x * d, g.y * d);
-            }
+        const float cx = gp.c.x, cb = gp.c.y, rho = gp.c.z;
+        // (0)
+        for (int it = threadIdx.x; it < 2 * N; it += T) {
+            const int b = it % N, h = it / N;   // column a = h M
+            const float4 g = __ldg(G + b * N + h * M);
+            const float af = h ? 0.f : (float)(-M), bf = (float)(b - M);
+            // on column M the mirror cell (a' = 0, -b') has the same D (D is even)
+            float d = cell_factor(g, af, bf, af * cx, cx, cb, rho, h == 0, h == 0 && b == 0);
+            if ((h * M + b) & 1) d = -d;
+            Z[b * LD + M + h] = make_float2(g.x * d, g.y * d);
         }
         __syncthreads();
-        // (1a) columns a in [0, M): R1-point DFT over b = n2 + R2 n1, twiddle
-        // exp(2 pi i n2 k1 / N), stored in place at rows n2 + R2 k1
+        // (1a) R1-point DFT over b = n2 + R2 n1, twiddle exp(2 pi i n2 k1 / N), to row k1 + R1 n2
 #pragma unroll 1
         for (int it = threadIdx.x; it < M * R2; it += T) {
             const int a = it % M, n2 = it / M;
+            const float af = (float)(a - M), lin0 = af * cx, b0 = (float)(n2 - M);
+            const float sg = ((a + n2) & 1) ? -1.f : 1.f;   // R2 is even
+            const float4 *g0 = G + n2 * N + a;
             float2 x[R1];
 #pragma unroll
             for (int n1 = 0; n1 < R1; ++n1) {
-                const int r = (n2 + R2 * n1) * LD;
-                float2 v = Z[r + a];
-                if (a == 0) {
-                    const float2 w = Z[r + M];
-                    v = make_float2(v.x - w.y, v.y + w.x);
+                const float4 g = __ldg(g0 + R2 * n1 * N);
+                const float d = sg * cell_factor(g, af, b0 + (float)(R2 * n1), lin0, cx, cb, rho, false, n1 == 0 && n2 == 0);
+                x[n1] = make_float2(g.x * d, g.y * d);
+            }
+            if (a == 0) {
+#pragma unroll
+                for (int n1 = 0; n1 < R1; ++n1) {
+                    const float2 *z = Z + (n2 + R2 * n1) * LD + M;
+                    x[n1] = make_float2(z[0].x - z[1].y, z[0].y + z[1].x);
                 }
-                x[n1] = v;
             }
             dft_reg<R1>(x);
 #pragma unroll
-            for (int k1 = 0; k1 < R1; ++k1) Z[(n2 + R2 * k1) * LD + a] = cmul(x[k1], tw[n2 * k1]);
+            for (int k1 = 0; k1 < R1; ++k1) Z[(k1 + R1 * n2) * LD + a] = cmul(x[k1], tw[n2 * k1]);
         }
         __syncthreads();
-        // (1b) R2-point DFT over n2 for each (a, k1); output rows j = k1 + R1 k2.  A part's
-        // reads all precede its writes; parts touch disjoint columns (column M belongs to
-        // the part holding column 0).
-#pragma unroll 1
-        for (int part = 0; part < P; ++part) {
-            constexpr int LA = M / P, NI = LA * R1, K = (NI + T - 1) / T;
-            float2 y[K][R2];
+        // (1b) R2-point DFT over n2 for each (a, k1), in place: output rows j = k1 + R1 k2
+#pragma unroll 2
+        for (int it = threadIdx.x; it < M * R1; it += T) {
+            const int a = it % M, k1 = it / M;
+            float2 *z = Z + k1 * LD;
+            float2 y[R2];
 #pragma unroll
-            for (int q = 0; q < K; ++q) {
-                const int it = threadIdx.x + q * T;
-                if (it < NI) {
-                    const int a = part * LA + it % LA, k1 = it / LA;
+            for (int n2 = 0; n2 < R2; ++n2) y[n2] = z[R1 * n2 * LD + a];
+            dft_reg<R2>(y);
+            if (a == 0) {
 #pragma unroll
-                    for (int n2 = 0; n2 < R2; ++n2) y[q][n2] = Z[(R2 * k1 + n2) * LD + a];
+                for (int k2 = 0; k2 < R2; ++k2) {
+                    z[R1 * k2 * LD] = make_float2(y[k2].x, 0.f);
+                    z[R1 * k2 * LD + M] = make_float2(y[k2].y, 0.f);
                 }
-            }
-            __syncthreads();
+            } else {
 #pragma unroll
-            for (int q = 0; q < K; ++q) {
-                const int it = threadIdx.x + q * T;
-                if (it < NI) {
-                    const int a = part * LA + it % LA, k1 = it / LA;
-                    dft_reg<R2>(y[q]);
-#pragma unroll
-                    for (int k2 = 0; k2 < R2; ++k2) {
-                        const int r = (k1 + R1 * k2) * LD;
-                        if (a == 0) {
-                            Z[r] = make_float2(y[q][k2].x, 0.f);
-                            Z[r + M] = make_float2(y[q][k2].y, 0.f);
-                        } else {
-                            Z[r + a] = y[q][k2];
-                        }
-                    }
-                }
+                for (int k2 = 0; k2 < R2; ++k2) z[R1 * k2 * LD + a] = y[k2];
             }
         }
         __syncthreads();
-        // (2a) rows j: C[k] for k = n2 + Q2 n1, Q1-point DFT over n1, twiddle
-        // exp(2 pi i n2 k1 / M) = tw[2 n2 k1], stored at k = n2 + Q2 k1 (parts = row ranges)
-#pragma unroll 1
-        for (int part = 0; part < P; ++part) {
-            constexpr int LJ = N / P, NI = LJ * Q2, K = (NI + T - 1) / T;
-            float2 c[K][Q1];
-#pragma unroll
-            for (int q = 0; q < K; ++q) {
-                const int it = threadIdx.x + q * T;
-                if (it < NI) {
-                    const int j = part * LJ + it % LJ, n2 = it / LJ;
-#pragma unroll
-                    for (int n1 = 0; n1 < Q1; ++n1) {
-                        const int k = n2 + Q2 * n1;
-                        const float2 zk = Z[j * LD + k], zm = Z[j * LD + M - k];
-                        const float2 e = make_float2(zk.x + zm.x, zk.y - zm.y);
-                        const float2 o = cmul(make_float2(zk.x - zm.x, zk.y + zm.y), tw[k]);
-                        c[q][n1] = make_float2(e.x - o.y, e.y + o.x);
-                    }
-                }
-            }
-            __syncthreads();
-#pragma unroll
-            for (int q = 0; q < K; ++q) {
-                const int it = threadIdx.x + q * T;
-                if (it < NI) {
-                    const int j = part * LJ + it % LJ, n2 = it / LJ;
-                    dft_reg<Q1>(c[q]);
-#pragma unroll
-                    for (int k1 = 0; k1 < Q1; ++k1) Z[j * LD + n2 + Q2 * k1] = cmul(c[q][k1], tw[2 * n2 * k1]);
-                }
-            }
-        }
-        __syncthreads();
-        // (2b) Q2-point DFT over n2 for each (j, k1): y[k1 + Q1 k2] = x[2n] + i x[2n+1],
-        // n = k1 + Q1 k2, stored at slot n of row j
-#pragma unroll 1
-        for (int part = 0; part < P; ++part) {
-            constexpr int LJ = N / P, NI = LJ * Q1, K = (NI + T - 1) / T;
-            float2 y[K][Q2];
-#pragma unroll
-            for (int q = 0; q < K; ++q) {
-                const int it = threadIdx.x + q * T;
-                if (it < NI) {
-                    const int j = part * LJ + it % LJ, k1 = it / LJ;
-#pragma unroll
-                    for (int n2 = 0; n2 < Q2; ++n2) y[q][n2] = Z[j * LD + Q2 * k1 + n2];
-                }
-            }
-            __syncthreads();
-#pragma unroll
-            for (int q = 0; q < K; ++q) {
-                const int it = threadIdx.x + q * T;
-                if (it < NI) {
-                    const int j = part * LJ + it % LJ, k1 = it / LJ;
-                    dft_reg<Q2>(y[q]);
-#pragma unroll
-                    for (int k2 = 0; k2 < Q2; ++k2) Z[j * LD + k1 + Q1 * k2] = y[q][k2];
-                }
-            }
-        }
-        __syncthreads();
-        // (3) out[j][2n], out[j][2n + 1] = (-1)^j (Re y[n], -Im y[n]), streamed
+        // (2) RW rows per warp and turn.  (2a) C[k] for k = n2 + Q2 n1, Q1-point DFT over n1, twiddle
+        // exp(2 pi i n2 k1 / M) = tw[2 n2 k1]; exchanged within the row at k1 Q2 + (n2 + k1) % Q2
+        // (banks).  (2b) Q2-point DFT over n2 for each k1: y[k1 + Q1 k2] = x[2n] + i x[2n+1].
+        const int n2 = lane % Q2;
         float *o = out + gp.off;
-        if ((gp.off & 1) == 0) {
-            for (int it = threadIdx.x; it < N * M; it += T) {
-                const int j = it / M, n = it % M;
-                const float2 y = Z[j * LD + n];
-                const float sg = (j & 1) ? -1.f : 1.f;
-                __stcs(reinterpret_cast<float2 *>(o + j * N + 2 * n), make_float2(sg * y.x, -sg * y.y));
+        const bool wide = (gp.off & 1) == 0;
+#pragma unroll 1
+        for (int j0 = (threadIdx.x / 32) * RW; j0 < N; j0 += (T / 32) * RW) {
+            float2 *z = Z + (j0 + lane / Q2) * LD;
+            float2 c[Q1];
+#pragma unroll
+            for (int n1 = 0; n1 < Q1; ++n1) {
+                const int k = n2 + Q2 * n1;
+                const float2 zk = z[k], zm = z[M - k];
+                const float2 e = make_float2(zk.x + zm.x, zk.y - zm.y);
+                const float2 od = cmul(make_float2(zk.x - zm.x, zk.y + zm.y), tw[k]);
+                c[n1] = make_float2(e.x - od.y, e.y + od.x);
             }
-        } else {
-            for (int it = threadIdx.x; it < N * M; it += T) {
-                const int j = it / M, n = it % M;
-                const float2 y = Z[j * LD + n];
+            dft_reg<Q1>(c);
+            __syncwarp();
+#pragma unroll
+            for (int k1 = 0; k1 < Q1; ++k1) z[k1 * Q2 + (n2 + k1) % Q2] = cmul(c[k1], tw[2 * n2 * k1]);
+            __syncwarp();
+#pragma unroll
+            for (int h = 0; h < Q1 / Q2; ++h) {
+                const int q = h * 32 + lane, k1 = q % Q1, j = j0 + q / Q1;
+                const float2 *zr = Z + j * LD + k1 * Q2;
+                float2 y[Q2];
+#pragma unroll
+                for (int i = 0; i < Q2; ++i) y[i] = zr[(i + k1) % Q2];
+                dft_reg<Q2>(y);
                 const float sg = (j & 1) ? -1.f : 1.f;
-                __stcs(o + j * N + 2 * n, sg * y.x);
-                __stcs(o + j * N + 2 * n + 1, -sg * y.y);
+                float *oj = o + j * N + 2 * k1;
+#pragma unroll
+                for (int k2 = 0; k2 < Q2; ++k2) {
+                    const float2 v = make_float2(sg * y[k2].x, -sg * y[k2].y);
+                    if (wide) {
+                        __stcs(reinterpret_cast<float2 *>(oj + 2 * Q1 * k2), v);
+                    } else {
+                        __stcs(oj + 2 * Q1 * k2, v.x);
+                        __stcs(oj + 2 * Q1 * k2 + 1, v.y);
+                    }
+                }
             }
         }
         __syncthreads();
@@ -643,19 +615,14 @@ __global__ void __launch_bounds__(kClThreads) __cluster_dims__(kClCtas, 1, 1)
                 const float4 q = Gc[it];
                 const float af = (float)(a - M), lin0 = af * cx, bf = (float)(b - M);
                 const float sg = ((a + b) & 1) ? -1.f : 1.f;
-                float e = sinc_fast(q.z * fmaf(bf, cb, lin0));
-                if (a == 0 || b == 0) {
-                    const float ma = a == 0 ? af : -af, mb = b == 0 ? bf : -bf;
-                    e = 0.5f * (e + sinc_fast(q.z * fmaf(ma, cx, mb * cb)));
-                }
-                const float d = sg * e * sinc_fast(q.w * rho);
+                const float d = sg * cell_factor(q, af, bf, lin0, cx, cb, rho, a == 0, b == 0);
                 Zc[b * LC + al] = make_float2(q.x * d, q.y * d);
             }
             if (c == 0)
                 for (int b = tid; b < N; b += T) {
                     const float4 q = Gc[N * CA + b];
                     const float bf = (float)(b - M);
-                    float d = sinc_fast(q.z * (bf * cb)) * sinc_fast(q.w * rho);
+                    float d = cell_factor(q, 0.f, bf, 0.f, cx, cb, rho, false, false);
                     if ((M + b) & 1) d = -d;
                     Zc[b * LC + CA] = make_float2(q.x * d, q.y * d);
                 }
