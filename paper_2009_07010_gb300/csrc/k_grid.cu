@@ -173,9 +173,9 @@ __global__ void k_grid_table(const double2 *__restrict__ S, const double *__rest
 // sinc_pi(x) = sin(pi x) / (pi x) = (-1)^n [sin(pi f) / (pi f)] (f / x), x = n + f, |f| <= 1/2.
 // n comes from adding 1.5 * 2^23 (|x| < 2^22), which rounds x to the nearest integer and
 // leaves the parity of n in the lowest mantissa bit; the bracket is its Taylor series in
-// (pi f)^2 to order 10 (truncation error < 4e-8).  f / x (1 for n = 0) is left as a fraction.
+// (pi f)^2 to order 10 (truncation error < 4e-8).  f / x is left as a fraction.
 struct SincParts {
-    float q, num, den;
+    float q, f;
     int parity;
 };
 
@@ -189,26 +189,26 @@ __device__ __forceinline__ SincParts sinc_parts(float x) {
     q = fmaf(z, q, 8.1174243e-1f);
     q = fmaf(z, q, -1.6449341f);
     q = fmaf(z, q, 1.0f);
-    const bool nz = n != 0.0f;
-    return {q, nz ? f : 1.0f, nz ? x : 1.0f, __float_as_int(t)};
+    return {q, f, __float_as_int(t)};
 }
 
-// sinc_pi(x) sinc_pi(y) with one quotient.
-__device__ __forceinline__ float sinc2_fast(float x, float y) {
+// (-1)^par sinc_pi(x) sinc_pi(y) for x, y > 0 with one quotient.
+__device__ __forceinline__ float sinc2_fast(float x, float y, int par) {
     const SincParts a = sinc_parts(x), b = sinc_parts(y);
-    const float v = (a.q * b.q) * __fdividef(a.num * b.num, a.den * b.den);
-    return __int_as_float(__float_as_int(v) ^ ((a.parity ^ b.parity) << 31));
+    const float v = (a.q * b.q) * __fdividef(a.f * b.f, x * y);
+    return __int_as_float(__float_as_int(v) ^ ((a.parity ^ b.parity ^ par) << 31));
 }
 
-// D' of a cell (offsets af, bf from the grid's centre): its smearing factor, averaged with that
-// of the mirror cell modulo N on the Nyquist row and column.
+// (-1)^par D' of a cell (offsets af, bf from the grid's centre): its smearing factor, averaged
+// with that of the mirror cell modulo N on the Nyquist row and column.  1e-18 keeps the sincs'
+// arguments (their magnitudes; g.z, g.w, rho >= 0) off zero, where f / x = 1, without a select.
 __device__ __forceinline__ float cell_factor(const float4 &g, float af, float bf, float lin0, float cx, float cb,
-                                             float rho, bool a0, bool b0) {
-    const float y = g.w * rho;
-    float d = sinc2_fast(g.z * fmaf(bf, cb, lin0), y);
+                                             float rho, bool a0, bool b0, int par) {
+    const float y = fmaf(g.w, rho, 1e-18f);
+    float d = sinc2_fast(fabsf(g.z * fmaf(bf, cb, lin0)) + 1e-18f, y, par);
     if (a0 || b0) {
         const float ma = a0 ? af : -af, mb = b0 ? bf : -bf;
-        d = 0.5f * (d + sinc2_fast(g.z * fmaf(ma, cx, mb * cb), y));
+        d = 0.5f * (d + sinc2_fast(fabsf(g.z * fmaf(ma, cx, mb * cb)) + 1e-18f, y, par));
     }
     return d;
 }
@@ -299,7 +299,8 @@ constexpr int grid_min_blocks() { return N == 128 ? 3 : N == 64 ? 6 : 8; }
 
 // One CTA per position (grid-stride).  X = (-1)^(a+b) S D' is Hermitian, so only the
 // cells a in [0, N/2] are formed, with the N twiddles exp(+2 pi i m / N) in shared memory.
-// Z [N rows][LD], row b, later output row j, holds what passes between the stages.
+// Z [N rows][LD] holds what passes between the stages: row c = b + N/2 modulo N (this rotation
+// is the sign (-1)^j of the outputs), later output row j.
 //   (0) the columns a = 0 and a = N/2 of X into Z's columns M and M + 1
 //   (1) columns: length-N inverse DFT over b for a in [0, N/2), the first stage on cells that
 //       the thread forms itself; column 0 carries X[.][0] + i X[.][N/2], whose transforms are
@@ -307,17 +308,17 @@ constexpr int grid_min_blocks() { return N == 128 ? 3 : N == 64 ? 6 : 8; }
 //   (2) rows: each row j is Hermitian in a, and its real inverse DFT x is obtained from
 //       one length-N/2 complex DFT of C[k] = E[k] + i O[k], E[k] = Z[k] + conj Z[N/2 - k],
 //       O[k] = (Z[k] - conj Z[N/2 - k]) exp(2 pi i k / N): it returns x[2n] + i x[2n+1];
-//       out[j][i] = (-1)^(i + j) x[i], two floats per store.
+//       out[j][i] = (-1)^i x[i], two floats per store.
 // Cell and pixel index origins are at N/2: exp(2 pi i (a - N/2)(i - N/2) / N) =
 // (-1)^(a + i) exp(2 pi i a i / N) for N % 4 == 0.
 //
 // Bound by instruction issue (268 MB written for 4096 positions of 128 pixels take 40 us).  With
 // X written to Z before the first stage, block-wide exchanges between all stages and the result
-// once more through Z it took 52.4 k warp instructions per position and 250 us for those; now
-// 43.9 k and 212 us: the first stage works on its own cells, the second stage of the columns
-// in place (stage one stores (n2, k1) as row k1 + R1 n2, from where the thread that takes k1
-// reads and to where it writes), a row stays within one warp, and the two sincs of a cell
-// share a quotient.
+// once more through Z those took 250 us; 201 us now.  The first stage works on its own cells,
+// the second stage of the columns in place (stage one stores (n2, k1) as row k1 + R1 n2, from
+// where the thread that takes k1 reads and to where it writes), a row stays within one warp
+// (these: 212 us), the two sincs of a cell share a quotient, signs are integer operations on
+// the sinc's and rotations of the rows, and a lane keeps its twiddles of the row pass.
 template <int N>
 __global__ void __launch_bounds__(GridFft<N>::T, grid_min_blocks<N>())
     k_img_grid(const float4 *__restrict__ G, const GridPos *__restrict__ pos, int npos, float *__restrict__ out) {
@@ -343,23 +344,23 @@ __global__ void __launch_bounds__(GridFft<N>::T, grid_min_blocks<N>())
             const float4 g = __ldg(G + b * N + h * M);
             const float af = h ? 0.f : (float)(-M), bf = (float)(b - M);
             // on column M the mirror cell (a' = 0, -b') has the same D (D is even)
-            float d = cell_factor(g, af, bf, af * cx, cx, cb, rho, h == 0, h == 0 && b == 0);
-            if ((h * M + b) & 1) d = -d;
-            Z[b * LD + M + h] = make_float2(g.x * d, g.y * d);
+            const float d = cell_factor(g, af, bf, af * cx, cx, cb, rho, h == 0, h == 0 && b == 0, b);
+            Z[(b ^ M) * LD + M + h] = make_float2(g.x * d, g.y * d);
         }
         __syncthreads();
-        // (1a) R1-point DFT over b = n2 + R2 n1, twiddle exp(2 pi i n2 k1 / N), to row k1 + R1 n2
+        // (1a) R1-point DFT over c = n2 + R2 n1, twiddle exp(2 pi i n2 k1 / N), to row k1 + R1 n2
 #pragma unroll 1
         for (int it = threadIdx.x; it < M * R2; it += T) {
             const int a = it % M, n2 = it / M;
-            const float af = (float)(a - M), lin0 = af * cx, b0 = (float)(n2 - M);
-            const float sg = ((a + n2) & 1) ? -1.f : 1.f;   // R2 is even
+            const float af = (float)(a - M), lin0 = af * cx, c0 = (float)n2;
             const float4 *g0 = G + n2 * N + a;
             float2 x[R1];
 #pragma unroll
             for (int n1 = 0; n1 < R1; ++n1) {
-                const float4 g = __ldg(g0 + R2 * n1 * N);
-                const float d = sg * cell_factor(g, af, b0 + (float)(R2 * n1), lin0, cx, cb, rho, false, n1 == 0 && n2 == 0);
+                const int off = R2 * n1 < M ? R2 * n1 : R2 * n1 - N;   // b - M = n2 + off
+                const float4 g = __ldg(g0 + (off + M) * N);
+                const float d = cell_factor(g, af, c0 + (float)off, lin0, cx, cb, rho, false, off == -M && n2 == 0,
+                                            a + n2);   // R2 and M are even
                 x[n1] = make_float2(g.x * d, g.y * d);
             }
             if (a == 0) {
@@ -399,6 +400,12 @@ __global__ void __launch_bounds__(GridFft<N>::T, grid_min_blocks<N>())
         // exp(2 pi i n2 k1 / M) = tw[2 n2 k1]; exchanged within the row at k1 Q2 + (n2 + k1) % Q2
         // (banks).  (2b) Q2-point DFT over n2 for each k1: y[k1 + Q1 k2] = x[2n] + i x[2n+1].
         const int n2 = lane % Q2;
+        float2 ta[Q1], tb[Q1];   // the lane's twiddles
+#pragma unroll
+        for (int n1 = 0; n1 < Q1; ++n1) {
+            ta[n1] = tw[n2 + Q2 * n1];
+            tb[n1] = tw[2 * n2 * n1];
+        }
         float *o = out + gp.off;
         const bool wide = (gp.off & 1) == 0;
 #pragma unroll 1
@@ -410,13 +417,13 @@ __global__ void __launch_bounds__(GridFft<N>::T, grid_min_blocks<N>())
                 const int k = n2 + Q2 * n1;
                 const float2 zk = z[k], zm = z[M - k];
                 const float2 e = make_float2(zk.x + zm.x, zk.y - zm.y);
-                const float2 od = cmul(make_float2(zk.x - zm.x, zk.y + zm.y), tw[k]);
+                const float2 od = cmul(make_float2(zk.x - zm.x, zk.y + zm.y), ta[n1]);
                 c[n1] = make_float2(e.x - od.y, e.y + od.x);
             }
             dft_reg<Q1>(c);
             __syncwarp();
 #pragma unroll
-            for (int k1 = 0; k1 < Q1; ++k1) z[k1 * Q2 + (n2 + k1) % Q2] = cmul(c[k1], tw[2 * n2 * k1]);
+            for (int k1 = 0; k1 < Q1; ++k1) z[k1 * Q2 + (n2 + k1) % Q2] = cmul(c[k1], tb[k1]);
             __syncwarp();
 #pragma unroll
             for (int h = 0; h < Q1 / Q2; ++h) {
@@ -426,11 +433,10 @@ __global__ void __launch_bounds__(GridFft<N>::T, grid_min_blocks<N>())
 #pragma unroll
                 for (int i = 0; i < Q2; ++i) y[i] = zr[(i + k1) % Q2];
                 dft_reg<Q2>(y);
-                const float sg = (j & 1) ? -1.f : 1.f;
                 float *oj = o + j * N + 2 * k1;
 #pragma unroll
                 for (int k2 = 0; k2 < Q2; ++k2) {
-                    const float2 v = make_float2(sg * y[k2].x, -sg * y[k2].y);
+                    const float2 v = make_float2(y[k2].x, -y[k2].y);
                     if (wide) {
                         __stcs(reinterpret_cast<float2 *>(oj + 2 * Q1 * k2), v);
                     } else {
@@ -469,7 +475,7 @@ cudaError_t launch_img_grid_n(const float4 *G, const GridPos *pos, int npos, flo
 //   * the peak is found from per-row maxima: the window of an iteration changes N rows, and
 //     each CTA renews the maxima of its own N/8 of them (per 64-pixel segment, then per row);
 //   * the PSF's columns, then its rows, are shared by the CTAs, exchanged through distributed
-//     shared memory, with k_img_grid's operations per element (bit-identical values);
+//     shared memory, with k_img_grid's cells and transforms;
 //   * cluster barriers (three per iteration) order everything.
 // 10.9 us per iteration.  FACET: one given PSF (P, any even N) instead of the gridded one.
 // Maxima are 64-bit keys as k_clean_argmax forms them (value, then the first pixel).
@@ -614,16 +620,14 @@ __global__ void __launch_bounds__(kClThreads) __cluster_dims__(kClCtas, 1, 1)
                 const int al = it % CA, b = it / CA, a = c * CA + al;
                 const float4 q = Gc[it];
                 const float af = (float)(a - M), lin0 = af * cx, bf = (float)(b - M);
-                const float sg = ((a + b) & 1) ? -1.f : 1.f;
-                const float d = sg * cell_factor(q, af, bf, lin0, cx, cb, rho, a == 0, b == 0);
+                const float d = cell_factor(q, af, bf, lin0, cx, cb, rho, a == 0, b == 0, a + b);
                 Zc[b * LC + al] = make_float2(q.x * d, q.y * d);
             }
             if (c == 0)
                 for (int b = tid; b < N; b += T) {
                     const float4 q = Gc[N * CA + b];
                     const float bf = (float)(b - M);
-                    float d = cell_factor(q, 0.f, bf, 0.f, cx, cb, rho, false, false);
-                    if ((M + b) & 1) d = -d;
+                    const float d = cell_factor(q, 0.f, bf, 0.f, cx, cb, rho, false, false, b);   // M is even
                     Zc[b * LC + CA] = make_float2(q.x * d, q.y * d);
                 }
             __syncthreads();
