@@ -85,13 +85,14 @@ extern "C" {
 
 /* ---- contraction algorithm (psf_opts_t.algo) ---------------------------- */
 /* PSF_ALGO_AUTO: positions of one cutout size (a multiple of 32 up to 256) take the
- * batched form when their group is large enough, the rest the per-cutout form.  The
- * batched form runs every such group of a call in one persistent launch per visibility
- * chunk (one CTA per SM pulling items from a work queue).  An autotuner, run on the first
- * batched call of a plan for each weight class (real / complex weights, FP16 / BF16) and
- * each cutout size first met, times probes over the first 2^19 visibilities (the call then
- * synchronizes its stream): per cutout size the group size from which the batched form
- * beats the per-cutout form.  The results are kept by the plan. */
+ * batched form in whole tiles of 128, and in a last, partial tile where that is cheaper
+ * than the per-cutout form, which takes the rest.  The batched form runs all tiles of a
+ * call in one persistent launch per visibility chunk (one CTA per SM pulling items from a
+ * work queue).  An autotuner, run on the first batched call of a plan for each weight class
+ * (real / complex weights, FP16 / BF16) and each cutout size first met, times probes over
+ * the first 2^19 visibilities (the call then synchronizes its stream): per cutout size the
+ * number of positions from which a tile of the batched form beats the per-cutout form.  The
+ * results are kept by the plan. */
 #define PSF_ALGO_AUTO 0   /* per-cutout form for small batches, batched otherwise */
 #define PSF_ALGO_CUTOUT 1 /* per-cutout separable form, split over visibilities  */
 

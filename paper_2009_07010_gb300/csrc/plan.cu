@@ -123,7 +123,7 @@ struct psf_plan_s {
     DevBuf err;          // int: device-side wait timeouts
     DevBuf queue;        // int: work queue of the persistent batched kernel
     // autotuner of the batched form, per weight class (bit 0 real weights, bit 1 BF16): per
-    // cutout size, the smallest group the batched form takes
+    // cutout size, the smallest remainder of whole tiles the batched form takes
     struct KrTune {
         std::map<int, int> min_group;
     };
