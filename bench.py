@@ -40,8 +40,8 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # profiles/k_psf_tc_meerkat64_1h_128px.md, per visibility (traffic is proportional to
 # K; the mean of the step's two launches: exact, fused uv + img), valid only for the
 # kernel source it was taken on.
-PROFILED_TRAFFIC = {"kernel_sha256_prefix": "86620fd584ed55e3",
-                    "bytes_per_vis": ((232.290816e6 + 3.294976e6) + (348.522496e6 + 0.410368e6)) / 2 / 14515200,
+PROFILED_TRAFFIC = {"kernel_sha256_prefix": "4b15b687bfefe165",
+                    "bytes_per_vis": ((232.459776e6 + 3.630848e6) + (348.445440e6 + 3.265024e6)) / 2 / 14515200,
                     "profile": "profiles/k_psf_tc_meerkat64_1h_128px.md"}
 
 
@@ -53,6 +53,10 @@ def profiled_traffic(nvis):
         return None
     return PROFILED_TRAFFIC["bytes_per_vis"] * nvis
 WORKLOAD = "meerkat64_4h_16ch_128px_single_cutout"
+# Tensor flops per position-pixel-visibility term of the batched contraction: a half plane of
+# pixels, two real products with complex weights and one with real weights (the border row and
+# column without a reflection, and padding, not counted).
+KR_FLOPS = {"exact": 2.0, "uv": 1.0, "img": 1.0}
 
 
 def load_peaks():
@@ -287,7 +291,7 @@ def measure_batched(psf, prec, steps=2, which="c4", profile_range=False):
     # 4 for the complex weights of the exact method, 2 for the real weights of the
     # approximations (one multiply-add per pixel-visibility term)
     per, total_ms = {}, 0.0
-    for m, fpt in (("exact", 4.0), ("uv", 2.0), ("img", 2.0)):
+    for m, fpt in KR_FLOPS.items():
         plan.forward(m, batch, out=out)
         torch.cuda.synchronize()
         plan.profile_read()
@@ -356,7 +360,7 @@ def measure_batched(psf, prec, steps=2, which="c4", profile_range=False):
             torch.cuda.synchronize()
             kms, nkc, _ = plan.profile_read()
             plan.profile_enable(False)
-            tf = 4.0 * K * len(sel) * N * N / (kms * 1e-3) / 1e12
+            tf = KR_FLOPS["exact"] * K * len(sel) * N * N / (kms * 1e-3) / 1e12
             per_size[f"{N}px"] = {"positions": int(len(sel)), "kernel_ms": kms, "kernel_tflops": tf,
                                   "kernel_frac_of_peak": tf / peaks["bf16_tflops"],
                                   "kernel_frac_of_sustained_peak":
@@ -374,7 +378,7 @@ def measure_batched(psf, prec, steps=2, which="c4", profile_range=False):
 
 # Executed warp-instructions per position of k_img_grid (ncu smsp__inst_executed.sum of one
 # launch / positions; profiles/k_img_grid_radial16384.md), for the kernel source below.
-PROFILED_GRID = {"kernel_sha256_prefix": "f623518e68ad870c", "inst_per_position": {128: 214640640 / 4096, 64: 44775424 / 4096}}
+PROFILED_GRID = {"kernel_sha256_prefix": "417e5b4aeba4702d", "inst_per_position": {128: 171083776 / 4096, 64: 32072192 / 4096}}
 
 
 def grid_inst_per_position(N):
@@ -682,8 +686,7 @@ def measure_c5(psf, prec, nrad=128, nang=128, ref="fp16"):
         raise RuntimeError("device-side wait timed out in the approximation workload")
     terms = K * bg.total_pixels()
     peaks, _ = load_peaks()
-    # algorithmic flops per term: 4 with the complex weights of the exact method, 2 with real weights
-    tfl = {m: (4.0 if m == "exact" else 2.0) * terms / (kms[m] * 1e-3) / 1e12 for m in ("exact", "uv", "img")}
+    tfl = {m: KR_FLOPS[m] * terms / (kms[m] * 1e-3) / 1e12 for m in ("exact", "uv", "img")}
     uvm, imm = res["uv"]["err_max"], res["img"]["err_max"]
     return {"workload": "meerkat64_8km_4h_256ch_avg4_radial16384_64px", "nvis": K, "positions": bg.npos,
             "grid": f"{nrad} radii 3 deg (a+1)/{nrad} x {nang} position angles, 64 px at 1.5 arcsec",
