@@ -40,7 +40,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # profiles/k_psf_tc_meerkat64_1h_128px.md, per visibility (traffic is proportional to
 # K; the mean of the step's two launches: exact, fused uv + img), valid only for the
 # kernel source it was taken on.
-PROFILED_TRAFFIC = {"kernel_sha256_prefix": "4b15b687bfefe165",
+PROFILED_TRAFFIC = {"kernel_sha256_prefix": "b15b687bfefe165d",
                     "bytes_per_vis": ((232.459776e6 + 3.630848e6) + (348.445440e6 + 3.265024e6)) / 2 / 14515200,
                     "profile": "profiles/k_psf_tc_meerkat64_1h_128px.md"}
 
