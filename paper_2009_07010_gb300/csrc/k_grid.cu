@@ -580,7 +580,9 @@ __global__ void __launch_bounds__(kClThreads) __cluster_dims__(kClCtas, 1, 1)
     int iter = st->iter;
     const int stop_at = min(max_iter, iter + chunk);
     bool done = st->done != 0;
-    __syncthreads();
+    // every CTA of the cluster runs before its shared memory is written by another (and this
+    // CTA's tables are filled)
+    cluster_barrier();
     while (!done && iter < stop_at) {
         // peak: every CTA takes the maximum of all row keys
         unsigned long long k = 0;
