@@ -476,7 +476,10 @@ cudaError_t launch_img_grid_n(const float4 *G, const GridPos *pos, int npos, flo
 //     each CTA renews the maxima of its own N/8 of them (per 64-pixel segment, then per row);
 //   * the PSF's columns, then its rows, are shared by the CTAs, exchanged through distributed
 //     shared memory, with k_img_grid's cells and transforms;
-//   * cluster barriers (three per iteration) order everything.
+//   * cluster barriers order everything.  Gridded: (1) the columns' results lie in the row
+//     owners' shared memory, (2) the rows are done (their centre is read remotely), (3) residual
+//     and keys are renewed; no CTA renews keys before (1) and (2), which follow everyone's
+//     reading of them.  One given PSF: a barrier between the reading and the renewal, and (3).
 // 10.9 us per iteration.  FACET: one given PSF (P, any even N) instead of the gridded one.
 // Maxima are 64-bit keys as k_clean_argmax forms them (value, then the first pixel).
 constexpr int kClCtas = 8, kClThreads = 256, kClSeg = 64;
@@ -607,6 +610,7 @@ __global__ void __launch_bounds__(kClThreads) __cluster_dims__(kClCtas, 1, 1)
         float scale;
         if (FACET) {
             scale = g / Pf[half * np + half];
+            cluster_barrier();   // every CTA has read the row keys before one renews its own
         } else {
             if (tid == 0) {
                 const double l0 = lc + (px - nl / 2) * cell, m0 = mc + (py - nm / 2) * cell;
