@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(GridFft<N>::T, grid_min_blocks<N>())
             tb[n1] = tw[2 * n2 * n1];
         }
         float *o = out + gp.off;
-        const bool wide = (gp.off & 1) == 0;
+        const bool wide = (reinterpret_cast<uintptr_t>(o) & 7) == 0;   // the caller's buffer may start at any float
 #pragma unroll 1
         for (int j0 = (threadIdx.x / 32) * RW; j0 < N; j0 += (T / 32) * RW) {
             float2 *z = Z + (j0 + lane / Q2) * LD;
