@@ -1534,7 +1534,7 @@ int psf_fwhm(psf_plan_t p, const psf_batch_t *b, const float *cutouts_dev, doubl
 
 int psf_img_grid_table(psf_plan_t p, int npix, double cell_rad, float *table_dev, void *stream) {
     if (!p || !table_dev || !(cell_rad > 0.0)) return PSF_EINVAL;
-    if (!img_grid_supported(npix)) return PSF_EUNSUPPORTED;
+    if (!img_grid_supported(npix) || (p->opts.flags & PSF_COMPLEX_OUT)) return PSF_EUNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     const float4 *G = nullptr;
     int s = grid_tables(p, npix, cell_rad, st, &G);
