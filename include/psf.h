@@ -229,10 +229,10 @@ int psf_approx_uv_img(psf_plan_t plan, const psf_batch_t *batch, float *out_uv_d
  * on uv cells; same arguments and output layout as psf_approx_img.  The grid of an
  * N x N cutout of pixel size cell is its N x N Fourier grid: cells du = dv = 1/(N cell),
  * cell (a, b) at ((a - N/2) du, (b - N/2) dv).  Position independent and built on the
- * first call for each (N, cell_rad, precision), then kept by the plan (that first call
- * synchronizes the stream): the effective PSF P (the cutout at the phase centre,
- * evaluated like psf_approx_img in the plan's precision), S = F{P}, and per cell the
- * W-weighted means of dt_k and Dnu_r / nu_r of the visibilities whose nearest cell,
+ * first call for each (N, cell_rad, precision), then kept by the plan until
+ * psf_plan_set_weights (the call that builds them synchronizes the stream): the effective
+ * PSF P (the cutout at the phase centre, evaluated like psf_approx_img in the plan's
+ * precision), S = F{P}, and per cell the W-weighted means of dt_k and Dnu_r / nu_r of the visibilities whose nearest cell,
  * modulo N, is the cell or its mirror (the means over all visibilities where none is).
  * Per position: D on every cell (the literal theta with PSF_IMG_LITERAL_THETA), one
  * inverse N x N FFT, FP32.  It differs from psf_approx_img by the gridding: D is taken at

@@ -111,11 +111,14 @@ struct psf_plan_s {
     std::vector<int64_t> h_bin_first, h_samp_first;
     int affine0 = 0;
     DevBuf samp_w, chan_win, bin_bl;
-    // gridded image-plane tables, one per (cutout size, pixel size, precision)
+    // gridded image-plane tables, one per (cutout size, pixel size, precision), of the weights
+    // they were built with (a count of psf_plan_set_weights calls)
+    int64_t weights_set = 0;
     struct Grid {
         int N = 0;
         double cell = 0;
         int prec = 0;
+        int64_t weights_set = -1;
         DevBuf G;   // float4 [N][N]
     };
     std::vector<std::unique_ptr<Grid>> grids;
@@ -424,6 +427,7 @@ int psf_plan_set_windows(psf_plan_t p, const float *tw, const float *cw) {
 int psf_plan_set_weights(psf_plan_t p, const float *w, void *stream) {
     if (!p) return PSF_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
+    p->weights_set++;   // the kept gridded tables are of other weights from here on
     if (w) {
         PSF_TRY(cudaMemcpyAsync(p->W.p, w, (size_t)p->nvis * sizeof(float), cudaMemcpyDeviceToDevice, st));
         return PSF_OK;
@@ -1203,21 +1207,29 @@ int run_forward_cplx(psf_plan_s *p, int method, const BatchHost &h, float *out, 
 }
 
 // Tables of the gridded image-plane form (Eq. 45, Algorithm 1) for one (N, cell,
-// precision), built on first use and kept by the plan: the effective PSF through the
+// precision), built on first use and kept by the plan until its weights are replaced (then
+// built again, into the same buffer, by the next call): the effective PSF through the
 // visibility-level path (Method 2 at the phase centre, where every decorrelation is 1),
 // its FP64 DFT, the per-cell mean intervals and fractional bandwidths, and the table.
 // The build synchronizes the stream (its temporaries are released on return).
 int grid_tables(psf_plan_s *p, int N, double cell, cudaStream_t st, const float4 **G) {
+    psf_plan_s::Grid *kept = nullptr;
     for (auto &g : p->grids)
-        if (g->N == N && g->cell == cell && g->prec == p->opts.prec) {
-            *G = (const float4 *)g->G.p;
-            return PSF_OK;
-        }
-    std::unique_ptr<psf_plan_s::Grid> g(new (std::nothrow) psf_plan_s::Grid());
-    if (!g) return PSF_ENOMEM;
-    g->N = N;
-    g->cell = cell;
-    g->prec = p->opts.prec;
+        if (g->N == N && g->cell == cell && g->prec == p->opts.prec) kept = g.get();
+    if (kept && kept->weights_set == p->weights_set) {
+        *G = (const float4 *)kept->G.p;
+        return PSF_OK;
+    }
+    std::unique_ptr<psf_plan_s::Grid> fresh;
+    if (!kept) {
+        fresh.reset(new (std::nothrow) psf_plan_s::Grid());
+        if (!fresh) return PSF_ENOMEM;
+        fresh->N = N;
+        fresh->cell = cell;
+        fresh->prec = p->opts.prec;
+    }
+    psf_plan_s::Grid *const g = kept ? kept : fresh.get();
+    g->weights_set = -1;   // until the build has succeeded
     const int64_t NN = (int64_t)N * N;
     DevBuf P, Y, S, acc;
     PSF_TRY(P.reserve(NN * sizeof(float)));
@@ -1243,8 +1255,9 @@ int grid_tables(psf_plan_s *p, int N, double cell, cudaStream_t st, const float4
                               (float4 *)g->G.p, st));
     if (p->prof) p->n_kernels += 4;
     PSF_TRY(cudaStreamSynchronize(st));
+    g->weights_set = p->weights_set;
     *G = (const float4 *)g->G.p;
-    p->grids.push_back(std::move(g));
+    if (fresh) p->grids.push_back(std::move(fresh));
     return PSF_OK;
 }
 
