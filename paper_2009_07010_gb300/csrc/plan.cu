@@ -548,9 +548,15 @@ constexpr int kKrMinGroup = 32;                     // positions of one size for
 // the count that minimises waves x (range + per-CTA overhead), in visibilities.  Small
 // observations are spread over the whole chip (ranges of 8192 and 4096 visibilities at
 // least left a 172 800-visibility cutout on 22 and 43 of the 152 SMs), and a count just
-// above a whole wave is avoided.
-int best_splits(int64_t base, int64_t K, int nsm, int64_t overhead, int64_t least) {
-    const int64_t most = std::max<int64_t>(1, std::min<int64_t>((K + least - 1) / least, 4 * (int64_t)nsm));
+// above a whole wave is avoided.  `bytes` are the partial sums of one range: those of all
+// ranges stay within kPartialBudget (an eighth of the weights' budget).  Large cutouts, whose
+// tiles fill the chip by themselves, would otherwise buy the last percents of a wave with
+// gigabytes (nine 4096-pixel cutouts on 58 M visibilities: 19 ranges, 11.5 GB); with four
+// ranges a wave's end costs at most a few percent there.
+constexpr int64_t kPartialBudget = int64_t(512) << 20;
+int best_splits(int64_t base, int64_t K, int nsm, int64_t overhead, int64_t least, int64_t bytes) {
+    const int64_t most = std::max<int64_t>(
+        1, std::min<int64_t>({(K + least - 1) / least, 4 * (int64_t)nsm, kPartialBudget / bytes}));
     int64_t best = 1, best_cost = INT64_MAX;
     for (int64_t n = 1; n <= most; ++n) {
         const int64_t cost = ((base * n + nsm - 1) / nsm) * ((K + n - 1) / n + overhead);
@@ -891,7 +897,7 @@ int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cud
                 for (int j0 = 0; j0 < N; j0 += tj)
                     for (int i0 = 0; i0 < N; i0 += ti) tiles.push_back(Tile{i, N, i0, j0, loc[i]});
             }
-            nsplit = best_splits((int64_t)tiles.size(), K, p->nsm, kFp32Overhead, kFp32Least);
+            nsplit = best_splits((int64_t)tiles.size(), K, p->nsm, kFp32Overhead, kFp32Least, 4 * chunk_px);
             kper = (int32_t)(((K + nsplit - 1) / nsplit + 31) / 32 * 32);
             nsplit = (int)((K + kper - 1) / kper);
         } else {
@@ -907,7 +913,7 @@ int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cud
                         base.push_back(TcItem{i, N, j0, i0, nc, 0, 0, 0, loc[i]});
                     }
             }
-            nsplit = best_splits((int64_t)base.size(), K, p->nsm, kTcOverhead, kTcLeast);
+            nsplit = best_splits((int64_t)base.size(), K, p->nsm, kTcOverhead, kTcLeast, 4 * chunk_px);
             kper = (int32_t)(((K + nsplit - 1) / nsplit + 31) / 32 * 32);
             nsplit = (int)((K + kper - 1) / kper);
             for (int sp = 0; sp < nsplit; ++sp)
@@ -1052,7 +1058,7 @@ int run_forward_uvimg(psf_plan_s *p, const psf_batch_t *b, float *out_uv, float 
             const int N = h.npix[c0 + i];
             base.push_back(TcItem{i, N, 0, 0, N, 0, 0, 0, loc[i]});
         }
-        int nsplit = best_splits(cn, K, p->nsm, kTcOverhead, kTcLeast);
+        int nsplit = best_splits(cn, K, p->nsm, kTcOverhead, kTcLeast, 8 * chunk_px);   // two halves
         const int32_t kper = (int32_t)(((K + nsplit - 1) / nsplit + 31) / 32 * 32);
         nsplit = (int)((K + kper - 1) / kper);
         for (int sp = 0; sp < nsplit; ++sp)
@@ -1140,7 +1146,7 @@ int run_forward_cplx(psf_plan_s *p, int method, const BatchHost &h, float *out, 
             ncols_max = std::max(ncols_max, nc);
             base.push_back(TcItem{i, N, 0, 0, nc, 0, 0, 0, loc[i]});
         }
-        int nsplit = best_splits(cn, K, p->nsm, kTcOverhead, kTcLeast);
+        int nsplit = best_splits(cn, K, p->nsm, kTcOverhead, kTcLeast, 8 * chunk_px);   // two halves
         const int32_t kper = (int32_t)(((K + nsplit - 1) / nsplit + 31) / 32 * 32);
         nsplit = (int)((K + kper - 1) / kper);
         for (int sp = 0; sp < nsplit; ++sp)
