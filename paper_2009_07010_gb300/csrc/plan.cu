@@ -745,8 +745,10 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
 // Autotuner of the batched form, run on the first batched call of a plan for each weight
 // class (real / complex weights, operand type) and cutout size N and cached in the plan: the
 // crossover between the forms.  Over a probe of the first kProbeVis visibilities it times
-// the per-cutout form for one more position and the batched form for one 128-position tile;
-// the batched form takes whole tiles, and a remainder of n positions when t_tile < n t_cutout.
+// the per-cutout form for one more position and the batched form for one 128-position tile,
+// each after an untimed run (the first launch of a kernel in a process loads it, on the host,
+// between the events); the batched form takes whole tiles, and a remainder of n positions when
+// t_tile < n t_cutout.
 constexpr int64_t kProbeVis = int64_t(1) << 19;
 
 int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cudaStream_t st, int64_t kmax = -1);
@@ -765,8 +767,17 @@ int kr_tune(psf_plan_s *p, int method, const BatchHost &hall, const std::vector<
         }
     DevBuf scratch;
     PSF_TRY(scratch.reserve((size_t)std::max<int64_t>(run, 1) * sizeof(float)));
-    const bool prof = p->prof;
-    p->prof = false;
+    // the plan's settings during the probes, put back on every way out
+    struct Settings {
+        psf_plan_s *p;
+        const bool prof;
+        const psf_opts_t opts;
+        explicit Settings(psf_plan_s *q) : p(q), prof(q->prof), opts(q->opts) { p->prof = false; }
+        ~Settings() {
+            p->prof = prof;
+            p->opts = opts;
+        }
+    } settings(p);
     int s = PSF_OK;
     // crossover per size: one position per-cutout against one 128-position tile batched
     for (const auto &g : cand) {
@@ -776,6 +787,7 @@ int kr_tune(psf_plan_s *p, int method, const BatchHost &hall, const std::vector<
         one[0].N = g.N;
         one[0].idx.assign(g.idx.begin(), g.idx.begin() + std::min<size_t>(g.idx.size(), 128));
         double t_tile = 0.0;
+        if ((s = run_kr(p, method, hs, one, (float *)scratch.p, st, probe))) break;   // untimed
         if ((s = run_kr(p, method, hs, one, (float *)scratch.p, st, probe, &t_tile))) break;
         // one more cutout in the per-cutout form: the difference of five and one, so that neither
         // launches nor the probe's short range count (with the time of a single cutout a tile was
@@ -788,7 +800,6 @@ int kr_tune(psf_plan_s *p, int method, const BatchHost &hall, const std::vector<
         b1.cell_rad = hall.cell;
         DevBuf cut;
         PSF_TRY(cut.reserve((size_t)5 * g.N * g.N * sizeof(float)));
-        const psf_opts_t saved = p->opts;
         p->opts.algo = PSF_ALGO_CUTOUT;
         cudaEvent_t ev[3] = {};
         for (auto &e : ev) PSF_TRY(cudaEventCreate(&e));
@@ -805,12 +816,11 @@ int kr_tune(psf_plan_s *p, int method, const BatchHost &hall, const std::vector<
         PSF_TRY(cudaEventElapsedTime(&t5, ev[0], ev[1]));
         PSF_TRY(cudaEventElapsedTime(&t1, ev[1], ev[2]));
         for (auto &e : ev) cudaEventDestroy(e);
-        p->opts = saved;
+        p->opts = settings.opts;
         const double t_cut = std::max(0.25 * (t5 - t1), 0.05 * t5);
         const double thr = t_cut > 0.0 ? t_tile / t_cut : 1e9;
         t.min_group[g.N] = (int)std::max(1.0, std::min(128.0, std::ceil(thr)));
     }
-    p->prof = prof;
     PSF_TRY(cudaStreamSynchronize(st));
     return s;
 }
