@@ -285,10 +285,12 @@ typedef struct {
  * [max_iter] or NULL: per iteration the peak pixel index y * nl + x and the subtracted
  * flux gain * I_D(l0).  *niter_out (host, may be NULL): iterations performed.  With
  * PSF_METHOD_IMG_GRID, and with PSF_CLEAN_FACET_PSF after the one PSF evaluation, the
- * loop runs inside a kernel and the host reads its record once per 1024 iterations; the
- * other methods read the peak record back each iteration to place the cutout.  Errors: PSF_EINVAL (sizes, gain, method, NULL
- * residual), PSF_EUNSUPPORTED (a cutout size the method does not support,
- * PSF_COMPLEX_OUT), and those of the PSF calls. */
+ * loop runs inside a kernel and the host reads its record once per 1024 iterations, or, for
+ * large windows of one PSF and for images of very many rows, as queued kernels with one
+ * reading per 64 iterations; the other methods read the peak record back each iteration to
+ * place the cutout.  Errors: PSF_EINVAL (sizes, gain, method, NULL residual),
+ * PSF_EUNSUPPORTED (a cutout size the method does not support, PSF_COMPLEX_OUT), and those
+ * of the PSF calls. */
 int psf_clean(psf_plan_t plan, const psf_clean_t *cfg, float *residual_dev, float *model_dev,
               int32_t *comp_pix_dev, float *comp_flux_dev, int32_t *niter_out, void *cuda_stream);
 /* (every pixel's direction must satisfy l^2 + m^2 < 1 where the loop places a cutout:

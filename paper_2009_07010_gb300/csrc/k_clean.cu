@@ -9,14 +9,18 @@
 //   k_clean_prep    one thread: decodes the key, applies the do-while test of the
 //                   algorithm (the first iteration always runs, later ones only while the
 //                   peak exceeds the threshold, at most max_iter), and writes the
-//                   iteration's record, peak pixel and value; clears the other key for
-//                   the next iteration
+//                   iteration's record: peak pixel and value, and the position record
+//                   the gridded PSF kernel reads; clears the other key for the next
+//                   iteration
 //   (the PSF cutout at l0, by any of the plan's methods)
 //   k_clean_sub     I_D -= gain I_D(l0) P / P(l0) on the N x N window around l0 (clipped
 //                   to the image); the model gains gain I_D(l0) at l0; the component is
 //                   recorded
-// The host reads the record each iteration to place the cutout.  (With the gridded PSF or
-// one PSF for the image the whole loop is one kernel, k_clean_loop in k_grid.cu.)
+// With the gridded PSF or one PSF for the image these serve the images and windows that are too
+// large for the one-kernel loop (k_clean_loop in k_grid.cu; the rule is in run_clean): every
+// kernel returns at once when the record says the loop has stopped, so a chunk of iterations
+// can be queued ahead and the host reads the record once per chunk.  With the other methods
+// the host reads the record each iteration to place the cutout.
 #include <cuda_runtime.h>
 
 #include "psf_internal.cuh"
@@ -61,7 +65,8 @@ __global__ void k_clean_argmax(const float *__restrict__ res, int64_t n, const C
 }
 
 __global__ void k_clean_prep(const unsigned long long *__restrict__ key, unsigned long long *__restrict__ key_next,
-                             CleanState *__restrict__ st, float threshold, int max_iter) {
+                             CleanState *__restrict__ st, int nl, int nm, double cell, double lc, double mc,
+                             float threshold, int max_iter, int literal) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     *key_next = 0ull;
     st->active = 0;
@@ -80,6 +85,12 @@ __global__ void k_clean_prep(const unsigned long long *__restrict__ key, unsigne
     st->active = 1;
     st->pix = pix;
     st->peak = peak;
+    const int x = pix % nl, y = pix / nl;
+    const double l0 = lc + (x - nl / 2) * cell, m0 = mc + (y - nm / 2) * cell;
+    const float rho = (float)sqrt(l0 * l0 + m0 * m0);
+    st->gpos.c = literal ? make_float4((float)-l0, (float)m0, rho, 0.f) : make_float4((float)m0, (float)-l0, rho, 0.f);
+    st->gpos.off = 0;
+    st->gpos.pad = 0;
 }
 
 __global__ void k_clean_sub(float *__restrict__ res, float *__restrict__ model, const float *__restrict__ P,
@@ -115,9 +126,10 @@ cudaError_t launch_clean_argmax(const float *res, int64_t n, const CleanState *s
     return cudaGetLastError();
 }
 
-cudaError_t launch_clean_prep(const unsigned long long *key, unsigned long long *key_next, CleanState *st,
-                              float threshold, int max_iter, cudaStream_t s) {
-    k_clean_prep<<<1, 32, 0, s>>>(key, key_next, st, threshold, max_iter);
+cudaError_t launch_clean_prep(const unsigned long long *key, unsigned long long *key_next, CleanState *st, int nl,
+                              int nm, double cell, double lc, double mc, float threshold, int max_iter, int literal,
+                              cudaStream_t s) {
+    k_clean_prep<<<1, 32, 0, s>>>(key, key_next, st, nl, nm, cell, lc, mc, threshold, max_iter, literal);
     return cudaGetLastError();
 }
 

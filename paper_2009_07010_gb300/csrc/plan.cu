@@ -1333,9 +1333,78 @@ int run_img_grid(psf_plan_s *p, const psf_batch_t *b, float *out, cudaStream_t s
     return PSF_OK;
 }
 
+// Whether an iteration of CLEAN with the gridded PSF (or, facet, one given PSF of N pixels) is
+// cheaper in the one-kernel loop on a cluster of eight CTAs (k_clean_loop) or as whole-chip
+// kernels (k_clean.cu).  The loop saves launches and the pass over the image, but it subtracts
+// its window with eight CTAs, scans the maxima of nm rows and renews a window row's maximum
+// from nl / 64 segments; the kernels pay 0.75 us per 10^6 pixels, three times that beyond L2.
+// The lines are fits to measured times per iteration (loop / kernels, us):
+//   one PSF   512^2 N = 64 4.4 / 6.9, 128 8.4 / 6.9, 512 74 / 12;  2048^2 N = 128 8.4 / 10.0, 192 17 / 11,
+//             1024 321 / 34;  4096^2 N = 192 16.6 / 19.2, 224 22.3 / 19.4;  8192^2 N = 512 103 / 117, 1024 330 / 146;
+//             16 columns x 262 144 rows N = 16 50 / 9.9;  262 144 x 16 N = 16 13.3 / 9.9, 128 27 / 9.9
+//   gridded   512^2 N = 16 4.7 / 8.8, 128 10.4 / 21.7;  8192^2 N = 128 11.5 / 125;
+//             16 columns x 262 144 rows N = 16 29.5 / 12.1
+bool clean_on_cluster(bool facet, int N, int nl, int nm) {
+    const double px = (double)nl * nm, N2 = (double)N * N, l2 = 32e6;   // pixels in L2
+    const int turns = (N + 63) / 64;                                     // window rows per warp
+    const double loop = facet ? 3.5 + 3.7e-4 * N2 + 2e-4 * nm + 3.7e-5 * nl * turns
+                              : 4.7 + 0.05 * N + 1e-4 * nm + 2.1e-5 * nl * turns;
+    const double chip = (facet ? 6.8 + 2.2e-5 * N2 : 7.0 + 0.117 * N) + 0.75e-6 * px + 1.5e-6 * std::max(0.0, px - l2);
+    return loop <= chip;
+}
+
+// The loop as whole-chip kernels queued in chunks: argmax, record, (gridded PSF at the peak,) window.
+int clean_chip(psf_plan_s *p, const psf_clean_t *c, const float4 *G, float *P, float *res, float *model, int32_t *cpix,
+               float *cflux, CleanState *sd, unsigned long long *key, int literal, CleanState &h, cudaStream_t st) {
+    constexpr int kChunk = 64;   // even: the alternating argmax keys repeat identically in every chunk
+    const int per_iter = G ? 4 : 3, N = c->psf_npix;
+    auto chunk = [&](cudaStream_t cs) -> cudaError_t {
+        for (int q = 0; q < kChunk; ++q) {
+            cudaError_t e = launch_clean_argmax(res, (int64_t)c->nl * c->nm, sd, key + (q & 1), p->nsm, cs);
+            if (e == cudaSuccess)
+                e = launch_clean_prep(key + (q & 1), key + ((q + 1) & 1), sd, c->nl, c->nm, c->cell_rad, c->l_c, c->m_c,
+                                      c->threshold, c->max_iter, literal, cs);
+            if (e == cudaSuccess && G) e = launch_img_grid(G, &sd->gpos, 1, N, P, p->nsm, cs);
+            if (e == cudaSuccess) e = launch_clean_sub(res, model, P, sd, c->nl, c->nm, N, c->gain, cpix, cflux, cs);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    };
+    // the first chunk on the caller's stream (it also sets the kernels' one-time attributes)
+    PSF_TRY(chunk(st));
+    if (p->prof) p->n_kernels += per_iter * kChunk;
+    PSF_TRY(cudaMemcpyAsync(&h, sd, sizeof(h), cudaMemcpyDeviceToHost, st));
+    PSF_TRY(cudaStreamSynchronize(st));
+    if (h.done) return PSF_OK;
+    // later chunks: the same launches captured once into a graph and replayed on a private stream
+    // (the caller's stream has drained; the call returns after the private stream has)
+    cudaStream_t cs = nullptr;
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t ge = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed);
+    if (e == cudaSuccess) {
+        const cudaError_t ec = chunk(cs);
+        e = cudaStreamEndCapture(cs, &g);
+        if (ec != cudaSuccess) e = ec;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
+    while (e == cudaSuccess && !h.done) {
+        e = cudaGraphLaunch(ge, cs);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&h, sd, sizeof(h), cudaMemcpyDeviceToHost, cs);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
+        if (p->prof) p->n_kernels += per_iter * kChunk;
+    }
+    if (ge) cudaGraphExecDestroy(ge);
+    if (g) cudaGraphDestroy(g);
+    if (cs) cudaStreamDestroy(cs);
+    if (e != cudaSuccess) cudaGetLastError();
+    return cuda_status(e);
+}
+
 // Hogbom CLEAN with position-dependent PSFs (Algorithm 2).  With the gridded PSF, or one PSF
-// for the whole image, the loop runs inside a kernel (k_clean_loop), many iterations per
-// launch; the other methods read the peak record back to place the cutout (k_clean.cu).
+// for the whole image, an iteration needs nothing from the host (clean_on_cluster chooses the
+// form); the other methods read the peak record back to place the cutout (k_clean.cu).
 int run_clean(psf_plan_s *p, const psf_clean_t *c, float *res, float *model, int32_t *cpix, float *cflux,
               int32_t *niter_out, cudaStream_t st) {
     if (!c || !res) return PSF_EINVAL;
@@ -1382,6 +1451,12 @@ int run_clean(psf_plan_s *p, const psf_clean_t *c, float *res, float *model, int
             int s = grid_tables(p, N, c->cell_rad, st, &G);
             if (s) return s;
         }
+        if (!clean_on_cluster(facet, N, c->nl, c->nm)) {
+            const int s = clean_chip(p, c, G, (float *)P.p, res, model, cpix, cflux, sd, key, literal, h, st);
+            if (s) return s;
+            if (niter_out) *niter_out = h.iter;
+            return PSF_OK;
+        }
         // kChunk iterations per launch (a few milliseconds); the loop record is read after each
         constexpr int kChunk = 1024;
         DevBuf keys;
@@ -1404,7 +1479,8 @@ int run_clean(psf_plan_s *p, const psf_clean_t *c, float *res, float *model, int
         b.cell_rad = c->cell_rad;
         for (;; ++t) {
             PSF_TRY(launch_clean_argmax(res, npx, sd, key + (t & 1), p->nsm, st));
-            PSF_TRY(launch_clean_prep(key + (t & 1), key + ((t + 1) & 1), sd, c->threshold, c->max_iter, st));
+            PSF_TRY(launch_clean_prep(key + (t & 1), key + ((t + 1) & 1), sd, c->nl, c->nm, c->cell_rad, c->l_c, c->m_c,
+                                      c->threshold, c->max_iter, literal, st));
             if (p->prof) p->n_kernels += 2;
             PSF_TRY(cudaMemcpyAsync(&h, sd, sizeof(h), cudaMemcpyDeviceToHost, st));
             PSF_TRY(cudaStreamSynchronize(st));
