@@ -15,6 +15,9 @@ through the public API from host buffers (plan upload, compute, read-back).
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 Under torchrun each rank evaluates its own cutout (positions shard with no
 collective; weak scaling).  --impl reference times the FP64 CPU oracle (rank 0).
+Standard output gets one JSON line, the headline; the side measurements (other precisions,
+batched and gridded workloads, CLEAN, facets, PSF widths, parity) go to standard error as one
+JSON object, `side_measurements`.
 """
 from __future__ import annotations
 
@@ -57,6 +60,13 @@ WORKLOAD = "meerkat64_4h_16ch_128px_single_cutout"
 # pixels, two real products with complex weights and one with real weights (the border row and
 # column without a reflection, and padding, not counted).
 KR_FLOPS = {"exact": 2.0, "uv": 1.0, "img": 1.0}
+
+
+def print_result(line, side):
+    """The headline as one short line on standard output (whoever keeps only the end of the
+    output keeps all of it), the side measurements as one line on standard error."""
+    print(json.dumps({"side_measurements": side}), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
 
 
 def load_peaks():
@@ -944,11 +954,10 @@ def main():
                 "dtype": {"tc_fp16": "f16", "tc_bf16": "bf16", "fp32": "f32", "tc_fp16x3": "f16x3",
                           "tc_bf16x3": "bf16x3"}[args.prec], "data": "synthetic",
                 "config": step_config(args, K, int(batch_g.npix[0])),
-                "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "fp32_plain": fp32, "precision_ladder": ladder,
-                "batched": batched, "batched_c3": batched_c3, "c5": c5, "img_grid": img_grid, "clean": clean, "fwhm": fwhm, "facets": facets,
-                "parity": parity,
-                "gpu_launches": int(nk), "clocks": clocks}
-        print(json.dumps(line), flush=True)
+                "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": int(nk), "clocks": clocks}
+        print_result(line, {"fp32_plain": fp32, "precision_ladder": ladder, "batched": batched, "batched_c3": batched_c3,
+                            "c5": c5, "img_grid": img_grid, "clean": clean, "fwhm": fwhm, "facets": facets,
+                            "parity": parity})
     plan.close()
     if dist:
         dist.destroy_process_group()
