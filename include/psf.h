@@ -92,7 +92,10 @@ extern "C" {
  * (real / complex weights, FP16 / BF16) and each cutout size first met, times probes over
  * the first 2^19 visibilities (the call then synchronizes its stream): per cutout size the
  * number of positions from which a tile of the batched form beats the per-cutout form.  The
- * results are kept by the plan. */
+ * results are kept by the plan.  Positions of one size in one call can thus go through either
+ * form, and which ones do depends on a timing: their rounding differs within the precision's
+ * tolerance.  PSF_DETERMINISTIC (or PSF_ALGO_CUTOUT) sends every position through the
+ * per-cutout form. */
 #define PSF_ALGO_AUTO 0   /* per-cutout form for small batches, batched otherwise */
 #define PSF_ALGO_CUTOUT 1 /* per-cutout separable form, split over visibilities  */
 

@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kFoldThreads, 2)
                                   2.0f * re_mul(B1, h2) + 3.0f * im_mul(B2, h3));
                     gm = B.inv * (re_mul(C0, h0) - im_mul(C1, h1) - re_mul(C2, h2) + im_mul(C3, h3) - im_mul(E0, h1) -
                                   2.0f * re_mul(E1, h2) + 3.0f * im_mul(E2, h3));
-                } else {   // also where far is not a number
+                } else {   // (fmaxf drops a NaN: such a sample is in the moments above, which are then NaN)
                     float wk[8], g8[8];   // copies: the arrays of the common path stay in registers
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {

@@ -10,8 +10,8 @@
 // j >= N/2, plus row 0 and the lower half of column 0, whose reflections lie outside the
 // cutout): two real GEMMs with K' = K each (one for real weights, O = 0) instead of one
 // with K' = 2K over all pixels, which is half the tensor work and half the twiddles per
-// cutout.  256 x 64^2 on 14.1 M visibilities, exact: contraction 49.8 ms -> 22 ms;
-// 512 mixed cutouts on 7.1 M visibilities, Method 1 (real): 167.5 ms -> 58 ms
+// cutout.  256 x 64^2 on 14.1 M visibilities, exact: contraction 49.8 ms -> 21.9 ms;
+// 512 mixed cutouts on 7.1 M visibilities, Method 1 (real): 167.5 ms -> 54.4 ms
 // (both with the contiguous weight stages and the unrolled issue loop below).
 //
 // One CTA computes a 128-position tile of 128 representative pixels (256 for real
@@ -336,10 +336,11 @@ __global__ void __launch_bounds__(kKrThreads, 1)
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(&full[grp]);
-                    // The uv slot is released only now: the stage's stores depend on the values read
-                    // from it.  Released right after the reading instruction, the slot was sometimes
-                    // refilled before a warp had its values (one 32-pixel run of one stage wrong in
-                    // up to half of the calls with many short items; none in 180 calls since).
+                    // The uv slot is released only now, behind the proxy fence above: its refill is a
+                    // write of the async proxy, and that fence is what orders the generic reads of the
+                    // slot before it.  Released right after the reads, with no fence between, one
+                    // 32-pixel run of one stage was wrong in up to half of the calls with many short
+                    // items; none of 2000 such calls since.
                     mbar_arrive(&in_empty[islot]);
                 }
             }

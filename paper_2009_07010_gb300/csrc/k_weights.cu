@@ -100,7 +100,7 @@ __device__ __forceinline__ void exact8_sums(const DevObs &o, float4 ub, int2 sm,
                 S[p][j] = make_float2(M[p][0].x - x * M[p][1].y - 0.5f * x * x * M[p][2].x + x * x * x / 6.0f * M[p][3].y,
                                       M[p][0].y + x * M[p][1].x - 0.5f * x * x * M[p][2].y - x * x * x / 6.0f * M[p][3].x);
             }
-        } else {   // also where far is not a number
+        } else {   // (fmaxf drops a NaN: such a sample is in the moments above, which are then NaN)
             // from the phasors of channels 3 and 4 outwards, e_{j+1} = 2 cos(step) e_j - e_{j-1}
 #pragma unroll
             for (int j = 0; j < 8; ++j) S[p][j] = make_float2(0.f, 0.f);
