@@ -750,6 +750,7 @@ int run_kr(psf_plan_s *p, int method, const BatchHost &h, const std::vector<KrGr
 // between the events); the batched form takes whole tiles, and a remainder of n positions when
 // t_tile < n t_cutout.
 constexpr int64_t kProbeVis = int64_t(1) << 19;
+constexpr int64_t kWarmVis = 4096;   // enough to have the batched kernels loaded
 
 int run_forward(psf_plan_s *p, int method, const psf_batch_t *b, float *out, cudaStream_t st, int64_t kmax = -1);
 
@@ -787,7 +788,7 @@ int kr_tune(psf_plan_s *p, int method, const BatchHost &hall, const std::vector<
         one[0].N = g.N;
         one[0].idx.assign(g.idx.begin(), g.idx.begin() + std::min<size_t>(g.idx.size(), 128));
         double t_tile = 0.0;
-        if ((s = run_kr(p, method, hs, one, (float *)scratch.p, st, probe))) break;   // untimed
+        if ((s = run_kr(p, method, hs, one, (float *)scratch.p, st, std::min(probe, kWarmVis)))) break;   // untimed
         if ((s = run_kr(p, method, hs, one, (float *)scratch.p, st, probe, &t_tile))) break;
         // one more cutout in the per-cutout form: the difference of five and one, so that neither
         // launches nor the probe's short range count (with the time of a single cutout a tile was
