@@ -195,8 +195,10 @@ int psf_plan_set_windows(psf_plan_t plan, const float *time_window, const float 
 /* Replace the visibility weights W_k (Eq. 6) used by later calls on this plan:
  * weights_dev is a device float32 [nvis] array in plan order, copied on cuda_stream
  * (stream-ordered: the array may be released once the stream has passed the call), or
- * NULL for the natural weights W_k = tavg[b] * favg.  Errors: PSF_EINVAL (NULL plan),
- * PSF_ECUDA (copy failure). */
+ * NULL for the natural weights W_k = tavg[b] * favg.  The tables of psf_approx_img_grid are
+ * built again by the next call that needs them (a replay of a captured psf_plan_set_weights
+ * is not seen by the plan: call it once more outside the graph before a gridded call).
+ * Errors: PSF_EINVAL (NULL plan), PSF_ECUDA (copy failure). */
 int psf_plan_set_weights(psf_plan_t plan, const float *weights_dev, void *cuda_stream);
 
 /* Replace the precision / flags / algorithm used by later calls on this plan. */
